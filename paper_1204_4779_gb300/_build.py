@@ -27,6 +27,7 @@ UNITS = {
     "stage_f32_d3.cu": ["-ftz=true"],
     "stage_f32_d3b.cu": ["-ftz=true"],
     "stage_f32_d12.cu": ["-ftz=true"],
+    "stage_rows.cu": ["-ftz=true"],
     "stage_f64.cu": ["--fmad=false"],
     "aux_kernels.cu": ["--fmad=false"],
     "hydro_abi.cu": [],
@@ -42,7 +43,7 @@ UNITS = {
     "tma_host.cu": [],
 }
 HEADERS = ["hydro_device.cuh", "stage_kernel.cuh", "stage_launch.cuh", "hydro_internal.h",
-           "batch_kernel.cuh", "tma.cuh"]
+           "batch_kernel.cuh", "tma.cuh", "pair_device.cuh", "row_kernel.cuh"]
 
 
 def nvcc() -> str:

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(kAuxThreads) cfl_kernel(const AuxT<T> A) {
     constexpr int NV = D + 2;
     // after a step that did not run (dt = 0: t reached t_end, or a failed state) there is
     // nothing to reduce; the same for every CTA
-    if (ADVANCE && !(__ldcg(&A.ctrl->dt) > 0.0)) return;
+    if (ADVANCE && !step_pending(A.ctrl)) return;
     T smax = T(0);
     bool bad = false;
     const long long stride = (long long)gridDim.x * blockDim.x;

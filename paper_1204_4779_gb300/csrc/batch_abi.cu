@@ -39,17 +39,46 @@ bool shapes_ok(int32_t n_grids, const int64_t *nx, const int64_t *ny) {
     return true;
 }
 
+// Columns of a work item: the tile's, or the stored columns of a strip (FP32 row tiles, one
+// strip per warp whatever the tile's width).
+int cols_of(int prec, int bx, int by) { return prec == HYDRO_F32 && by == 1 ? hydro::kBatchStripCols : bx; }
+
+// Rows of an FP32 strip's work item when the variant names none: the least (rows to march
+// through, each item's prologue counted as two rows, over the GPU's resident warps) plus 0.3 item
+// of tail.  Sizes of the workspace follow from it, so the warps are those of a 152-SM
+// GPU (16 each) wherever it is asked.  Measured on GB300, ms per step at 8 / 16 / 32 / 64 / 96
+// rows, chosen marked: 4096 grids of 32-512 cells a side 3.29 / 2.97 / 2.75 / 2.61* / 2.60;
+// 1000 of 32-128: 0.174 / 0.170* / 0.181 / 0.198 / 0.236; 64 of 100-400: 0.098 / 0.096 / 0.103 /
+// 0.145 / 0.161 (12, chosen: 0.094).
+int strip_rows(int32_t n_grids, const int64_t *nx, const int64_t *ny) {
+    static const int kRows[] = {2, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96};
+    int best = 0;
+    double best_cost = 0.0;
+    for (int m : kRows) {
+        double work = 0.0;
+        for (int g = 0; g < n_grids; ++g) {
+            const double strips = (double)((nx[g] + hydro::kBatchStripCols - 1) / hydro::kBatchStripCols);
+            work += strips * ((double)ny[g] + 2.0 * (double)((ny[g] + m - 1) / m));
+        }
+        const double cost = work / (152.0 * 16.0) + 0.3 * (m + 2.0);
+        if (best == 0 || cost < best_cost) best = m, best_cost = cost;
+    }
+    return best;
+}
+
 // Tile of the batch kernels and the rows of one work item (the tile height, or for row tiles,
 // tile_y = 1, the march along y).
-// Default: FP32 row tiles of 32 columns marching 32 rows (4096 uneven grids: 24.3 G
-// cell-updates/s against 16.4 G for the 32 x 8 tile kernel); FP64 the 32 x 8 tiles.
-void tile_of(int prec, const hydro_variant_t *v, int *bx, int *by, int *rows) {
+// Default: FP32 row tiles (strips of 60 columns, one per warp); FP64 the 32 x 8 tiles.
+void tile_of(int prec, const hydro_variant_t *v, int32_t n_grids, const int64_t *nx,
+             const int64_t *ny, int *bx, int *by, int *rows) {
     *bx = 32;
     *by = prec == HYDRO_F32 ? 1 : 8;
     if (v && v->tile_x) *bx = v->tile_x;
     if (v && v->tile_y) *by = v->tile_y;
     *rows = *by;
-    if (*by == 1) *rows = (v && v->march > 0) ? v->march : 32;
+    if (*by == 1)
+        *rows = (v && v->march > 0) ? v->march
+                                    : (prec == HYDRO_F32 ? strip_rows(n_grids, nx, ny) : 32);
 }
 
 bool tile_ok(int prec, int bx, int by, const hydro_variant_t *v) {
@@ -109,6 +138,7 @@ struct hydro_batch {
     int periodic[2] = {1, 1};
     int tile_x = 32, tile_y = 8;
     int rows = 8;  // rows of a work item
+    int cols = 32; // its columns
     int n_blocks = 1;
     cudaStream_t stream = nullptr;
     cudaStream_t cap = nullptr;
@@ -154,6 +184,7 @@ BatchLaunch launch_args(const hydro_batch *b, const hydro_state_t *s, int kind, 
     L.tile_x = b->tile_x;
     L.tile_y = b->tile_y;
     L.march = b->rows;
+    L.cols = b->cols;
     return L;
 }
 
@@ -254,9 +285,9 @@ int hydro_batch_workspace_bytes(int32_t n_grids, const int64_t *nx, const int64_
     if (!bytes_out || !shapes_ok(n_grids, nx, ny)) return HYDRO_EINVAL;
     if (prec != HYDRO_F32 && prec != HYDRO_F64) return HYDRO_EINVAL;
     int bx, by, rows;
-    tile_of(prec, variant, &bx, &by, &rows);
+    tile_of(prec, variant, n_grids, nx, ny, &bx, &by, &rows);
     if (!tile_ok(prec, bx, by, variant)) return HYDRO_EUNSUPPORTED;
-    *bytes_out = batch_layout(n_grids, nx, ny, prec, bx, rows).total;
+    *bytes_out = batch_layout(n_grids, nx, ny, prec, cols_of(prec, bx, by), rows).total;
     return HYDRO_OK;
 }
 
@@ -273,9 +304,10 @@ int hydro_batch_create(int32_t n_grids, const int64_t *nx, const int64_t *ny, do
         if (bc[a] != HYDRO_BC_PERIODIC && bc[a] != HYDRO_BC_OUTFLOW) return HYDRO_EINVAL;
     if (((uintptr_t)workspace) % kAlign) return HYDRO_EINVAL;
     int bx, by, rows;
-    tile_of(prec, variant, &bx, &by, &rows);
+    tile_of(prec, variant, n_grids, nx, ny, &bx, &by, &rows);
     if (!tile_ok(prec, bx, by, variant)) return HYDRO_EUNSUPPORTED;
-    const BatchLayout lay = batch_layout(n_grids, nx, ny, prec, bx, rows);
+    const int cols = cols_of(prec, bx, by);
+    const BatchLayout lay = batch_layout(n_grids, nx, ny, prec, cols, rows);
     if (workspace_bytes < lay.total) return HYDRO_EINVAL;
     if (lay.n_items >= (1LL << 31)) return HYDRO_EUNSUPPORTED;
 
@@ -295,6 +327,7 @@ int hydro_batch_create(int32_t n_grids, const int64_t *nx, const int64_t *ny, do
     b->tile_x = bx;
     b->tile_y = by;
     b->rows = rows;
+    b->cols = cols;
     b->stream = static_cast<cudaStream_t>(stream);
     b->ws = static_cast<unsigned char *>(workspace);
     b->ctrl = reinterpret_cast<Ctrl *>(b->ws + lay.ctrl_off);
@@ -321,11 +354,11 @@ int hydro_batch_create(int32_t n_grids, const int64_t *nx, const int64_t *ny, do
         G.dr[1] = 1.0 / (double)ny[g];
         G.inv_dr[0] = (float)(1.0 / G.dr[0]);
         G.inv_dr[1] = (float)(1.0 / G.dr[1]);
-        const int tx = (G.nx + bx - 1) / bx, ty = (G.ny + rows - 1) / rows;
+        const int tx = (G.nx + cols - 1) / cols, ty = (G.ny + rows - 1) / rows;
         G.ntiles = tx * ty;
         G.first_item = (int)hi.size();
         for (int j = 0; j < ty; ++j)
-            for (int i = 0; i < tx; ++i) hi.push_back(BatchItem{g, i * bx, j * rows, 0});
+            for (int i = 0; i < tx; ++i) hi.push_back(BatchItem{g, i * cols, j * rows, 0});
         b->offsets[(size_t)g] = off;
         off += nx[g] * ny[g];
     }

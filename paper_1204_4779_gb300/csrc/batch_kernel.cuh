@@ -16,6 +16,7 @@
 
 #include "hydro_device.cuh"
 #include "hydro_internal.h"
+#include "row_kernel.cuh"
 #include "stage_kernel.cuh"
 
 namespace hydro {
@@ -34,6 +35,8 @@ template <class T> struct BatchArgs {
     double t_end, cfl;
     int periodic[2];
     int rows;   // rows of a work item: the tile height, or the march of row tiles
+    int cols;   // columns of a work item
+    int vec;    // strip kernels: every plane starts on an 8-byte boundary
     Gas<T> gas;
 };
 
@@ -92,10 +95,9 @@ __global__ void __launch_bounds__(BX * BY, (MinBlocks<T, BX * BY>::value))
         const BatchItem W = A.items[it];
         const BatchGrid R = A.grids[W.g];
         Ctrl *ctrl = A.ctrl + W.g;
-        const double dt = __ldcg(&ctrl->dt);
-        if (!(dt > 0.0)) continue;  // this grid takes no step (same for the whole CTA)
-        const T cx = T(__ldcg(&ctrl->coef[STAGE - 1][0]));
-        const T cy = T(__ldcg(&ctrl->coef[STAGE - 1][1]));
+        if (!step_pending(ctrl)) continue;  // this grid takes no step (same for the whole CTA)
+        const T cx = step_coef<T>(ctrl, STAGE, 0);
+        const T cy = step_coef<T>(ctrl, STAGE, 1);
         const int nx = R.nx, ny = R.ny;
         const int x = W.x0 + tx, y = W.y0 + ty;
         const bool active = (x < nx) && (y < ny);
@@ -173,7 +175,7 @@ __global__ void __launch_bounds__(BX * BY, (MinBlocks<T, BX * BY>::value))
     }
 }
 
-// Row tiles: a work item is a strip of BX columns of one grid and a chunk of `rows` rows,
+// FP64 row tiles: a work item is a strip of BX columns of one grid and a chunk of `rows` rows,
 // advanced by the single-grid kernels' per-tile code (stage_tile) marching along y, with the
 // same per-tile CFL slot as the tile kernel above.  Items are claimed dynamically: CTA b takes
 // item b first, then the next unclaimed item from a counter (items differ in size -- ragged
@@ -197,10 +199,9 @@ __global__ void __launch_bounds__(BX, (MinBlocks<T, BX, OCC>::value))
         const BatchItem W = A.items[it];
         const BatchGrid R = A.grids[W.g];
         Ctrl *ctrl = A.ctrl + W.g;
-        const double dt = __ldcg(&ctrl->dt);
-        if (!(dt > 0.0)) continue;  // this grid takes no step (same for the whole CTA)
-        const T cx = T(__ldcg(&ctrl->coef[STAGE - 1][0]));
-        const T cy = T(__ldcg(&ctrl->coef[STAGE - 1][1]));
+        if (!step_pending(ctrl)) continue;  // this grid takes no step (same for the whole CTA)
+        const T cx = step_coef<T>(ctrl, STAGE, 0);
+        const T cy = step_coef<T>(ctrl, STAGE, 1);
         StageArgs<T> V;  // the grid as a single-grid problem
         for (int k = 0; k < 4; ++k) {
             V.uin[k] = A.uin[k] + R.off;
@@ -233,6 +234,55 @@ __global__ void __launch_bounds__(BX, (MinBlocks<T, BX, OCC>::value))
     }
 }
 
+// FP32 row tiles: an item is a strip of kStripCells columns of one grid and a chunk of `rows`
+// rows, advanced by one warp (row_kernel.cuh), which claims its items by itself.  4096 grids of
+// 32-512 cells a side (121 M cells): 4.46 ms per step with the shared-memory row tiles of 32
+// columns, 2.61 ms so (46 G cell-updates/s; bound by instruction issue).  CTAs of four warps
+// against one: 2.61 / 2.86 ms.
+template <int STAGE>
+__global__ void __launch_bounds__(kRowThreads, 4) batch_strip_kernel(const BatchArgs<float> A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t ring = smem_u32(smem_raw) + warp * RowRing<STAGE>::bytes;
+    const PairGas G = pair_gas(A.gas);
+    auto claim_next = [&]() -> int {
+        unsigned int c = 0;
+        if (lane == 0) c = atomicAdd(A.claim + (STAGE - 1), 1u);
+        return (int)(gridDim.x * warps + __shfl_sync(0xffffffffu, c, 0));
+    };
+    for (int it = blockIdx.x * warps + warp; it < A.n_items; it = claim_next()) {
+        const BatchItem W = A.items[it];
+        const BatchGrid R = A.grids[W.g];
+        const Ctrl *ctrl = A.ctrl + W.g;
+        if (!step_pending(ctrl)) continue;  // this grid takes no step (same for the whole warp)
+        RowGrid V;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            V.uin[k] = A.uin[k] + R.off;
+            V.ubase[k] = A.ubase[k] + R.off;
+            V.uout[k] = A.uout[k] + R.off;
+        }
+        V.nx = R.nx, V.ny = R.ny;
+        V.px = A.periodic[0], V.py = A.periodic[1];
+        V.order = 2, V.riemann = 0;
+        V.cx = step_coef<float>(ctrl, STAGE, 0);
+        V.cy = step_coef<float>(ctrl, STAGE, 1);
+        V.inv_dr[0] = R.inv_dr[0], V.inv_dr[1] = R.inv_dr[1];
+        float smax = 0.0f, vmin = 1.0f;
+        const int ye = min(W.y0 + A.rows, R.ny);
+        // packed grids start at any cell: 64-bit accesses where this grid's rows allow them
+        if (A.vec && R.nx % 2 == 0 && R.off % 2 == 0)
+            row_strip<STAGE, (STAGE == 2), true, false>(V, G, W.x0 - 2, W.y0, ye, ring, smax, vmin);
+        else
+            row_strip<STAGE, (STAGE == 2), false, false>(V, G, W.x0 - 2, W.y0, ye, ring, smax, vmin);
+        if constexpr (STAGE == 2) {
+            unsigned int m = __float_as_uint(vmin > 0.0f ? smax : NAN);
+            m = __reduce_max_sync(0xffffffffu, m);  // bit patterns: NaN > inf > finite
+            if (lane == 0) A.tile_sig[it] = __uint_as_float(m);
+        }
+    }
+}
+
 // Per-grid start of a step call: control block of grid g reset, time t0[g] (or 0).
 static __global__ void batch_init_kernel(Ctrl *ctrl, const BatchGrid *grids, int n_grids,
                                   const double *t0, double t_end, double cfl, unsigned int *claim) {
@@ -258,27 +308,29 @@ __global__ void __launch_bounds__(BX * BY) batch_cfl_kernel(const BatchArgs<T> A
     for (int it = blockIdx.x; it < A.n_items; it += gridDim.x) {
         const BatchItem W = A.items[it];
         const BatchGrid R = A.grids[W.g];
-        const int x = W.x0 + tx;
+        const int xe = min(W.x0 + A.cols, R.nx), ye = min(W.y0 + A.rows, R.ny);
         T smax = T(0);
         bool bad = false;
-        for (int y = W.y0 + ty; y < W.y0 + A.rows && y < R.ny && x < R.nx; y += BY) {
-            const long long i = R.off + (long long)y * R.nx + x;
-            T u[4], v[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) u[k] = A.uin[k][i];
-            prim_of_cons<T, 2>(u, v, A.gas);
-            T s = T(0);
-            if constexpr (Arith<T>::exact) {
-                const T cs = sqrt(A.gas.g * v[3] / v[0]);
-                s = s + (fabs(v[1]) + cs) / R.dr[0];
-                s = s + (fabs(v[2]) + cs) / R.dr[1];
-            } else {
-                const T cs = Arith<float>::sqrt_(A.gas.g * v[3] * Arith<float>::rcp(v[0]));
-                s = fmaf(fabsf(v[1]) + cs, R.inv_dr[0], s);
-                s = fmaf(fabsf(v[2]) + cs, R.inv_dr[1], s);
+        for (int y = W.y0 + ty; y < ye; y += BY) {
+            for (int x = W.x0 + tx; x < xe; x += BX) {
+                const long long i = R.off + (long long)y * R.nx + x;
+                T u[4], v[4];
+    #pragma unroll
+                for (int k = 0; k < 4; ++k) u[k] = A.uin[k][i];
+                prim_of_cons<T, 2>(u, v, A.gas);
+                T s = T(0);
+                if constexpr (Arith<T>::exact) {
+                    const T cs = sqrt(A.gas.g * v[3] / v[0]);
+                    s = s + (fabs(v[1]) + cs) / R.dr[0];
+                    s = s + (fabs(v[2]) + cs) / R.dr[1];
+                } else {
+                    const T cs = Arith<float>::sqrt_(A.gas.g * v[3] * Arith<float>::rcp(v[0]));
+                    s = fmaf(fabsf(v[1]) + cs, R.inv_dr[0], s);
+                    s = fmaf(fabsf(v[2]) + cs, R.inv_dr[1], s);
+                }
+                smax = (s > smax || s != s) ? s : smax;
+                bad |= !(v[0] > T(0)) || !(v[3] > T(0));
             }
-            smax = (s > smax || s != s) ? s : smax;
-            bad |= !(v[0] > T(0)) || !(v[3] > T(0));
         }
         const T m = block_max<T, NT>(bad ? T(NAN) : smax, sRed);
         if (threadIdx.x == 0) A.tile_sig[it] = m;
@@ -312,14 +364,14 @@ __global__ void __launch_bounds__(256) batch_finalize_kernel(const BatchArgs<T> 
         const U other = __shfl_xor_sync(0xffffffffu, m, o);
         m = other > m ? other : m;
     }
+    Ctrl *c = A.ctrl + g;
     if (lane == 0) {
-        Ctrl *c = A.ctrl + g;
         if constexpr (sizeof(T) == 4)
             c->sig32 = (unsigned int)m;
         else
             c->sig64 = (unsigned long long)m;
-        finalize_dt<T>(c, ADVANCE);
     }
+    finalize_dt<T>(c, ADVANCE);
 }
 
 // Conserved totals of every grid in FP64: one CTA per grid, fixed per-thread strides and a
@@ -366,6 +418,12 @@ template <class T> BatchArgs<T> make_batch_args(const BatchLaunch &L) {
     A.periodic[0] = L.periodic[0];
     A.periodic[1] = L.periodic[1];
     A.rows = L.tile_y == 1 ? L.march : L.tile_y;
+    A.cols = L.cols;
+    A.vec = 1;
+    for (int k = 0; k < 4; ++k)
+        A.vec &= reinterpret_cast<uintptr_t>(L.uin[k]) % 8 == 0 &&
+                 reinterpret_cast<uintptr_t>(L.ubase[k]) % 8 == 0 &&
+                 reinterpret_cast<uintptr_t>(L.uout[k]) % 8 == 0;
     A.gas = make_gas<T>(L.gamma);
     return A;
 }
@@ -379,6 +437,10 @@ template <class T, int BX, int BY, int OCC> struct BatchKernels<T, BX, BY, OCC, 
     static constexpr auto s1 = batch_row_kernel<T, BX, 1, OCC>;
     static constexpr auto s2 = batch_row_kernel<T, BX, 2, OCC>;
 };
+template <int BX, int OCC> struct BatchKernels<float, BX, 1, OCC, true> {
+    static constexpr auto s1 = batch_strip_kernel<1>;
+    static constexpr auto s2 = batch_strip_kernel<2>;
+};
 
 // Dispatch for one precision: kind 0 = init, 1 = CFL pass, 2/3 = RK stage 1/2, 4 = totals;
 // prepare_only sets the shared-memory attribute and returns the resident CTAs per SM of the
@@ -389,23 +451,27 @@ cudaError_t batch_dispatch_tile(const BatchLaunch &L, cudaStream_t st, int kind,
     using S = StageShape<T, 2, BX, BY>;
     constexpr bool rows = (BY == 1);  // row tiles march along y
     // the tile kernel keeps one primitive and one flux plane; row tiles use stage_tile's two each
-    const size_t smem = sizeof(T) * (size_t)((rows ? 2 : 1) * 4 * (S::PL + S::NF) + 2 * (S::NT / 32));
+    constexpr bool strips = rows && sizeof(T) == 4;  // one strip per warp, a ring each
+    constexpr size_t tile_smem = sizeof(T) * (size_t)((rows ? 2 : 1) * 4 * (S::PL + S::NF) + 2 * (S::NT / 32));
+    constexpr int nt = strips ? kRowThreads : S::NT;
+    constexpr size_t smem1 = strips ? RowRing<1>::bytes * (size_t)(nt / 32) : tile_smem;
+    constexpr size_t smem2 = strips ? RowRing<2>::bytes * (size_t)(nt / 32) : tile_smem;
     using K = BatchKernels<T, BX, BY, OCC, rows>;
     const auto s1 = K::s1, s2 = K::s2;
     if (prepare_only) {
-        cudaError_t e = cudaFuncSetAttribute(s1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(s1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(s2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = cudaFuncSetAttribute(s2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
         if (e == cudaSuccess && blocks_per_sm)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, s2, S::NT, smem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, s2, nt, smem2);
         return e;
     }
     const BatchArgs<T> A = make_batch_args<T>(L);
     switch (kind) {
         case 0: batch_init_kernel<<<(L.n_grids + 255) / 256, 256, 0, st>>>(A.ctrl, A.grids, L.n_grids, A.t0, A.t_end, A.cfl, A.claim); break;
-        case 1: batch_cfl_kernel<T, BX, BY><<<L.n_blocks, S::NT, 0, st>>>(A); break;
-        case 2: s1<<<L.n_blocks, S::NT, smem, st>>>(A); break;
-        case 3: s2<<<L.n_blocks, S::NT, smem, st>>>(A); break;
+        case 1: batch_cfl_kernel<T, strips ? 32 : BX, strips ? nt / 32 : BY><<<L.n_blocks, nt, 0, st>>>(A); break;
+        case 2: s1<<<L.n_blocks, nt, smem1, st>>>(A); break;
+        case 3: s2<<<L.n_blocks, nt, smem2, st>>>(A); break;
         case 4: batch_totals_kernel<T><<<L.n_grids, 256, 0, st>>>(A, L.n_grids); break;
         case 5: batch_finalize_kernel<T, false><<<(L.n_grids * 32 + 255) / 256, 256, 0, st>>>(A, L.n_grids); break;
         case 6: batch_finalize_kernel<T, true><<<(L.n_grids * 32 + 255) / 256, 256, 0, st>>>(A, L.n_grids); break;

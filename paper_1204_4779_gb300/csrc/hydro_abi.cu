@@ -303,6 +303,7 @@ struct hydro_ctx {
     double lo[3] = {0, 0, 0};
     void *frame[5] = {};
     hydro_variant_t var = {};
+    int strip_rows = 0;      // FP32 row tiles without a named march: rows of a warp
     Layout lay = {};
     unsigned char *ws = nullptr;
     Ctrl *ctrl = nullptr;
@@ -348,6 +349,7 @@ hydro::StageLaunch stage_args(const hydro_ctx *c, const hydro_state_t *s, int st
         L.dr[a] = c->dr[a];
     }
     L.march = c->var.march;
+    L.rows = c->strip_rows;
     L.tile_x = c->var.tile_x;
     L.tile_y = c->var.tile_y;
     L.prefetch = c->var.staging == 2 ? 0 : (c->var.staging == 3 ? 2 : 1);
@@ -683,12 +685,14 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
             return HYDRO_EUNSUPPORTED;  // the ring's int indices
     }
     const bool rows = grid->dim == 2 && var.tile_y == 1;
+    int strip_rows = 0;
     if ((grid->dim == 3 || rows) && prec == HYDRO_F32 && !(variant && variant->march)) {
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
             var.march = rows ? default_march_rows(grid->n, var, sms)
                              : default_march_3d(grid->n, var, sms);
+        if (rows) strip_rows = hydro::default_strip_rows(grid->n[0], grid->n[1], sms);
     }
     const Layout lay = layout_for(grid->dim, grid->n, ncell, prec, var.manifest);
     if (workspace_bytes < lay.total) return HYDRO_EINVAL;
@@ -722,6 +726,7 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
     c->gamma = gamma;
     c->cfl = cfl;
     c->var = var;
+    c->strip_rows = strip_rows;
     c->lay = lay;
     c->ws = static_cast<unsigned char *>(workspace);
     c->ctrl = reinterpret_cast<Ctrl *>(c->ws + lay.ctrl_off);

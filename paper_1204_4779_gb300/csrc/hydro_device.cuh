@@ -39,6 +39,8 @@ struct Ctrl {
     double totals[5];       // output of the totals reduction
     double dr[3];           // cell sizes (set by the host with t, t_end, cfl)
     double coef[2][3];      // (dt/2)/dr_a and dt/dr_a of the next step, for RK stages 1 and 2
+    float coef32[2][3];     // the same rounded to FP32 (a conversion costs a kernel's every warp
+                            // as much as an FP64 operation)
 };
 static_assert(sizeof(Ctrl) <= 256, "the control block has 256 bytes in every workspace");
 
@@ -346,48 +348,69 @@ template <> __device__ __forceinline__ void push_signal<double>(Ctrl *c, double 
     atomicMax(&c->sig64, (unsigned long long)__double_as_longlong(s));
 }
 
-// Run by one thread of the last CTA of a reduction launch.  `advance`: a step with dt = c->dt
-// has just completed (no step ran if that dt is 0, e.g. once t reached t_end).  Then dt of the
-// next step = cfl / max signal, clipped onto t_end.
+// Whether the control block holds a step to take (dt > 0; dt is never NaN), without an FP64
+// comparison.
+__device__ __forceinline__ bool step_pending(const Ctrl *c) {
+    return __ldcg(reinterpret_cast<const long long *>(&c->dt)) > 0;
+}
+// AddFlux coefficient of RK stage `stage` (1 or 2) along axis a.
+template <class T> __device__ __forceinline__ T step_coef(const Ctrl *c, int stage, int a) {
+    if constexpr (sizeof(T) == 4)
+        return __ldcg(&c->coef32[stage - 1][a]);
+    else
+        return __ldcg(&c->coef[stage - 1][a]);
+}
+
+// Run by one whole warp of the last CTA of a reduction launch.  `advance`: a step with
+// dt = c->dt has just completed (no step ran if that dt is 0, e.g. once t reached t_end).  Then
+// dt of the next step = cfl / max signal, clipped onto t_end.  Lane 0 sets dt; the six
+// coefficients are divided one per lane (an FP64 division takes a warp about 600 cycles however
+// few lanes take part, and every step waits for this).
 template <class T> __device__ void finalize_dt(Ctrl *c, bool advance) {
     volatile Ctrl *vc = c;
-    if (advance && vc->dt > 0.0) {
-        const double dt = vc->dt;
-        vc->t = vc->clipped ? vc->t_end : vc->t + dt;
-        vc->dt_last = dt;
-        vc->steps = vc->steps + 1;
-    }
-    const double s = take_signal<T>(c);
-    const double t = vc->t, t_end = vc->t_end;
+    const int lane = threadIdx.x & 31;
     double dt = 0.0;
-    int clipped = 0;
-    if (!(s <= 1.7976931348623157e308) || !(s > 0.0)) {  // NaN, inf or no signal
-        atomicOr(&c->status, STATUS_NONFINITE);
-    } else if (vc->status == 0u) {
-        dt = vc->cfl / s;
-        if (t_end > 0.0) {
-            if (t >= t_end) {
-                dt = 0.0;
-            } else if (dt >= t_end - t) {
-                dt = t_end - t;
-                clipped = 1;
+    if (lane == 0) {
+        if (advance && vc->dt > 0.0) {
+            const double d = vc->dt;
+            vc->t = vc->clipped ? vc->t_end : vc->t + d;
+            vc->dt_last = d;
+            vc->steps = vc->steps + 1;
+        }
+        const double s = take_signal<T>(c);
+        const double t = vc->t, t_end = vc->t_end;
+        int clipped = 0;
+        if (!(s <= 1.7976931348623157e308) || !(s > 0.0)) {  // NaN, inf or no signal
+            atomicOr(&c->status, STATUS_NONFINITE);
+        } else if (vc->status == 0u) {
+            dt = vc->cfl / s;
+            if (t_end > 0.0) {
+                if (t >= t_end) {
+                    dt = 0.0;
+                } else if (dt >= t_end - t) {
+                    dt = t_end - t;
+                    clipped = 1;
+                }
             }
         }
+        if (atomicOr(&c->status, 0u) != 0u) dt = 0.0;
+        vc->dt = dt;
+        vc->clipped = clipped;
     }
-    if (atomicOr(&c->status, 0u) != 0u) dt = 0.0;
-    vc->dt = dt;
-    vc->clipped = clipped;
+    dt = __shfl_sync(0xffffffffu, dt, 0);
     // AddFlux coefficients of both stages, in the order of Eq. eqAddFlux: (c dt) / dr_a
-    for (int a = 0; a < 3; ++a) {
-        vc->coef[0][a] = (0.5 * dt) / vc->dr[a];
-        vc->coef[1][a] = dt / vc->dr[a];
+    if (lane < 6) {
+        const int st = lane / 3, a = lane - 3 * st;
+        const double q = (st == 0 ? 0.5 * dt : dt) / vc->dr[a];
+        vc->coef[st][a] = q;
+        vc->coef32[st][a] = (float)q;
     }
     __threadfence();
 }
 
 // Block-wide max of a non-negative value (NaN propagates as the largest bit pattern), then
 // one atomic per CTA; the last of `nblocks` contributions (0: every CTA of the launch)
-// finalises dt.  Call from all threads.
+// finalises dt.  Call from all threads of the CTA (NT of them; NT = 0: blockDim.x).
 template <class T, int NT>
 __device__ __forceinline__ void reduce_signal_and_finalize(Ctrl *ctrl, T smax, bool bad,
                                                            bool advance, T *sred,
@@ -409,24 +432,27 @@ __device__ __forceinline__ void reduce_signal_and_finalize(Ctrl *ctrl, T smax, b
     U *sb = reinterpret_cast<U *>(sred);
     if (lane == 0) sb[warp] = bits;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        U m = 0;
+    if (warp == 0) {
+        unsigned int last = 0;
+        if (lane == 0) {
+            U m = 0;
 #pragma unroll 1
-        for (int w = 0; w < NT / 32; ++w) m = sb[w] > m ? sb[w] : m;
-        T bm;
-        if constexpr (sizeof(T) == 4)
-            bm = __uint_as_float(m);
-        else
-            bm = __longlong_as_double((long long)m);
-        push_signal<T>(ctrl, bm);
-        if (anybad) atomicOr(&ctrl->status, STATUS_NONFINITE);
-        __threadfence();
-        if (nblocks == 0) nblocks = gridDim.x * gridDim.y * gridDim.z;
-        const unsigned int prev = atomicAdd(&ctrl->blocks_done, 1u);
-        if (prev == nblocks - 1) {
+            for (int w = 0; w < (NT ? NT : (int)blockDim.x) / 32; ++w) m = sb[w] > m ? sb[w] : m;
+            T bm;
+            if constexpr (sizeof(T) == 4)
+                bm = __uint_as_float(m);
+            else
+                bm = __longlong_as_double((long long)m);
+            push_signal<T>(ctrl, bm);
+            if (anybad) atomicOr(&ctrl->status, STATUS_NONFINITE);
+            __threadfence();
+            if (nblocks == 0) nblocks = gridDim.x * gridDim.y * gridDim.z;
+            last = atomicAdd(&ctrl->blocks_done, 1u) == nblocks - 1;
+        }
+        if (__shfl_sync(0xffffffffu, last, 0)) {
             __threadfence();
             finalize_dt<T>(ctrl, advance);
-            atomicExch(&ctrl->blocks_done, 0u);
+            if (lane == 0) atomicExch(&ctrl->blocks_done, 0u);
         }
     }
 }

@@ -19,6 +19,7 @@ struct StageLaunch {
     int n[3];
     int periodic[3];
     int march;
+    int rows;           // FP32 row tiles of dim 2: rows a warp marches through (0: march)
     int tile_x, tile_y;
     int prefetch;       // dim 3: 1 = next plane's loads one plane ahead, 0 = at staging,
                         // 2 = planes staged by TMA (FP32 tiles compiled with it)
@@ -44,6 +45,10 @@ cudaError_t stage_f32_d1(const StageLaunch &L, cudaStream_t st, bool prepare_onl
 cudaError_t stage_f32_d2(const StageLaunch &L, cudaStream_t st, bool prepare_only);
 cudaError_t stage_f32_d3(const StageLaunch &L, cudaStream_t st, bool prepare_only);
 cudaError_t stage_f64(int dim, const StageLaunch &L, cudaStream_t st, bool prepare_only);
+// The FP32 row tiles of dim 2 (stage_rows.cu), and the rows a warp of theirs marches through by
+// default on an nx x ny grid.
+cudaError_t stage_rows_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only);
+int default_strip_rows(long long nx, long long ny, int sm_count);
 
 // Compiled tile shapes (both_pf: both staging depths compiled).
 struct TileShape {
@@ -111,6 +116,7 @@ cudaError_t launch_exchange(const ExchangeLaunch &L, cudaStream_t st);
 cudaError_t launch_analytic_frame(const AnalyticLaunch &L, int stage, cudaStream_t st);
 
 // ---- batched 2D grids (batch_kernel.cuh) ----
+constexpr int kBatchStripCols = 60;  // columns of an FP32 row tile's work item
 struct BatchItem {  // one tile of one grid
     int g, x0, y0, pad;
 };
@@ -140,6 +146,7 @@ struct BatchLaunch {
     int n_blocks;        // persistent grid size
     int tile_x, tile_y;  // tile_y = 1: row tiles, which march along y
     int march;           // rows of a row tile's work item
+    int cols;            // columns of a work item
 };
 // kind: 0 init, 1 CFL pass (tile maxima), 2 RK stage 1, 3 RK stage 2 (+ tile maxima),
 // 4 per-grid totals, 5 per-grid dt from the tile maxima (first dt of a call), 6 the same after

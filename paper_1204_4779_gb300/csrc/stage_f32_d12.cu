@@ -1,5 +1,5 @@
 // FP32 RK-stage kernels, dims 1 and 2 (compiled with FMA contraction): one-plane tiles, and in
-// dim 2 also row tiles that march along y.
+// dim 2 row tiles that march along y (stage_rows.cu).
 #include "stage_launch.cuh"
 
 namespace hydro {
@@ -15,10 +15,8 @@ cudaError_t stage_f32_d2(const StageLaunch &L, cudaStream_t st, bool prepare_onl
     HYDRO_STAGE_CASE(float, 2, 64, 4, false)
     HYDRO_STAGE_CASE(float, 2, 16, 16, false)
     HYDRO_STAGE_CASE(float, 2, 32, 16, false)
-    // row tiles: BX cells of x, marching along y
-    HYDRO_STAGE_CASE(float, 2, 64, 1, true)
-    HYDRO_STAGE_CASE(float, 2, 128, 1, true)
-    HYDRO_STAGE_CASE(float, 2, 256, 1, true)
+    // row tiles: strips of 64 columns per warp, marching along y
+    if (L.tile_y == 1) return stage_rows_f32(L, st, prepare_only);
     return cudaErrorInvalidValue;
 }
 

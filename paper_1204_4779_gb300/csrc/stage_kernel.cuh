@@ -768,12 +768,11 @@ __global__ void __launch_bounds__(BX * BY, (MinBlocks<T, BX * BY, OCC>::value))
     T *const sRed = reinterpret_cast<T *>(smem_raw) + 2 * S::NV * S::PL + 2 * S::NV * S::NF;
 
     Ctrl *ctrl = A.ctrl;
-    const double dt = __ldcg(&ctrl->dt);
-    if (!(dt > 0.0)) return;  // uniform over the grid: no step to take
+    if (!step_pending(ctrl)) return;  // uniform over the grid: no step to take
     // (c dt)/dr_a, computed once per step in FP64 by the dt finaliser
-    const T cx = T(__ldcg(&ctrl->coef[STAGE - 1][0]));
-    const T cy = (GM::IN >= 2) ? T(__ldcg(&ctrl->coef[STAGE - 1][1])) : T(0);
-    const T cz = GM::march ? T(__ldcg(&ctrl->coef[STAGE - 1][GM::MA])) : T(0);
+    const T cx = step_coef<T>(ctrl, STAGE, 0);
+    const T cy = (GM::IN >= 2) ? step_coef<T>(ctrl, STAGE, 1) : T(0);
+    const T cz = GM::march ? step_coef<T>(ctrl, STAGE, GM::MA) : T(0);
     const int x0 = blockIdx.x * BX;
     const int y0 = (GM::IN >= 2) ? blockIdx.y * BY : 0;
     const int zb = GM::march ? ((int)blockIdx.z + A.zchunk0) * A.march : 0;
@@ -804,11 +803,10 @@ __global__ void __launch_bounds__(BX * BY, (MinBlocks<T, BX * BY, OCC>::value))
     __shared__ int s_item;
 
     Ctrl *ctrl = A.ctrl;
-    const double dt = __ldcg(&ctrl->dt);
-    if (!(dt > 0.0)) return;  // uniform over the grid: no step to take (and nothing claimed)
-    const T cx = T(__ldcg(&ctrl->coef[STAGE - 1][0]));
-    const T cy = (GM::IN >= 2) ? T(__ldcg(&ctrl->coef[STAGE - 1][1])) : T(0);
-    const T cz = T(__ldcg(&ctrl->coef[STAGE - 1][GM::MA]));
+    if (!step_pending(ctrl)) return;  // uniform over the grid: no step to take (and nothing claimed)
+    const T cx = step_coef<T>(ctrl, STAGE, 0);
+    const T cy = (GM::IN >= 2) ? step_coef<T>(ctrl, STAGE, 1) : T(0);
+    const T cz = step_coef<T>(ctrl, STAGE, GM::MA);
     T smax = T(0);
     bool bad = false;
     constexpr bool CFL = STAGE == 2 && FUSED;
@@ -846,11 +844,10 @@ __global__ void __launch_bounds__(BX * BY, (MinBlocks<T, BX * BY, OCC>::value))
     T *const sRed = reinterpret_cast<T *>(smem_raw) + 2 * S::NV * S::PL + 2 * S::NV * S::NF;
 
     Ctrl *ctrl = A.ctrl;
-    const double dt = __ldcg(&ctrl->dt);
-    if (!(dt > 0.0)) return;  // uniform over the grid: no step to take
-    const T cx = T(__ldcg(&ctrl->coef[STAGE - 1][0]));
-    const T cy = T(__ldcg(&ctrl->coef[STAGE - 1][1]));
-    const T cz = T(__ldcg(&ctrl->coef[STAGE - 1][2]));
+    if (!step_pending(ctrl)) return;  // uniform over the grid: no step to take
+    const T cx = step_coef<T>(ctrl, STAGE, 0);
+    const T cy = step_coef<T>(ctrl, STAGE, 1);
+    const T cz = step_coef<T>(ctrl, STAGE, 2);
     const int x0 = blockIdx.x * BX;
     const int y0 = blockIdx.y * BY;
     const int zb = ((int)blockIdx.z + A.zchunk0) * A.march;
@@ -891,11 +888,10 @@ __global__ void __launch_bounds__(kPassThreads) addflux_kernel(const StageArgs<T
     constexpr int D = 3, NV = 5;
     __shared__ T sRed[2 * kPassThreads / 32];
     Ctrl *ctrl = A.ctrl;
-    const double dt = __ldcg(&ctrl->dt);
-    if (!(dt > 0.0)) return;
-    const T cx = T(__ldcg(&ctrl->coef[STAGE - 1][0]));
-    const T cy = T(__ldcg(&ctrl->coef[STAGE - 1][1]));
-    const T cz = T(__ldcg(&ctrl->coef[STAGE - 1][2]));
+    if (!step_pending(ctrl)) return;
+    const T cx = step_coef<T>(ctrl, STAGE, 0);
+    const T cy = step_coef<T>(ctrl, STAGE, 1);
+    const T cz = step_coef<T>(ctrl, STAGE, 2);
     const int nx = A.n[0], ny = A.n[1], nz = A.n[2];
     const long long plane = (long long)nx * ny, ncell = plane * nz;
     T smax = T(0);
