@@ -2,7 +2,8 @@
 
 Each translation unit compiles in parallel into ``_build/``; the shared library lands next to
 this file.  FP64 translation units use ``--fmad=false`` (one correctly rounded IEEE operation
-per arithmetic operation); FP32 ones keep FMA contraction and flush denormals.
+per arithmetic operation); so do the FP32 ones, whose fused multiply-adds are written out, and
+which flush denormals.
 
     python -m paper_1204_4779_gb300._build [--force] [--verbose]
 """
@@ -22,17 +23,21 @@ OUT_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libhydro.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
+# FP32 kernels flush denormals and spell out every fused multiply-add: without contraction by the
+# compiler a cell's result does not depend on which kernel computed it
+FP32 = ["-ftz=true", "--fmad=false"]
 # translation unit -> extra flags
 UNITS = {
-    "stage_f32_d3.cu": ["-ftz=true"],
-    "stage_f32_d3b.cu": ["-ftz=true"],
-    "stage_f32_d12.cu": ["-ftz=true"],
-    "stage_rows.cu": ["-ftz=true"],
+    "stage_f32_d3.cu": FP32,
+    "stage_f32_d3b.cu": FP32,
+    "stage_f32_d12.cu": FP32,
+    "stage_rows.cu": FP32,
+    "stage_strip3.cu": FP32,
     "stage_f64.cu": ["--fmad=false"],
     "aux_kernels.cu": ["--fmad=false"],
     "hydro_abi.cu": [],
     "static_step.cu": [],
-    "batch_f32.cu": ["-ftz=true"],
+    "batch_f32.cu": FP32,
     "batch_f64.cu": ["--fmad=false"],
     "batch_abi.cu": [],
     "mlp.cu": [],
@@ -43,7 +48,8 @@ UNITS = {
     "tma_host.cu": [],
 }
 HEADERS = ["hydro_device.cuh", "stage_kernel.cuh", "stage_launch.cuh", "hydro_internal.h",
-           "batch_kernel.cuh", "tma.cuh", "pair_device.cuh", "row_kernel.cuh"]
+           "batch_kernel.cuh", "tma.cuh", "pair_device.cuh", "row_kernel.cuh",
+           "strip3_kernel.cuh"]
 
 
 def nvcc() -> str:

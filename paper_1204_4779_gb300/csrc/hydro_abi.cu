@@ -231,6 +231,12 @@ int default_march_rows(const int64_t n[3], const hydro_variant_t &v, int sm_coun
     return choose_march(strips, n[1], resident_slots(v, sm_count), 2.0, kMarch, 5, 16);
 }
 
+// The variants the 3D strip kernels run (stage_strip3.cu).
+bool strips3(int prec, int dim, const hydro_variant_t &v) {
+    return prec == HYDRO_F32 && dim == 3 && v.tile_x == 16 && v.tile_y == 8 && v.staging == 1 &&
+           v.manifest == 1;
+}
+
 // Resolve a (possibly partial) variant against the defaults; false if not compiled.
 bool resolve_variant(int prec, int dim, const hydro_variant_t *in, hydro_variant_t *out) {
     default_variant(prec, dim, out);
@@ -304,6 +310,8 @@ struct hydro_ctx {
     void *frame[5] = {};
     hydro_variant_t var = {};
     int strip_rows = 0;      // FP32 row tiles without a named march: rows of a warp
+    int march = 1;           // planes of a chunk: the variant's, or where it names none and the
+                             // 3D strip kernels run, their own choice
     Layout lay = {};
     unsigned char *ws = nullptr;
     Ctrl *ctrl = nullptr;
@@ -348,7 +356,7 @@ hydro::StageLaunch stage_args(const hydro_ctx *c, const hydro_state_t *s, int st
         L.periodic[a] = c->periodic[a];
         L.dr[a] = c->dr[a];
     }
-    L.march = c->var.march;
+    L.march = c->march;
     L.rows = c->strip_rows;
     L.tile_x = c->var.tile_x;
     L.tile_y = c->var.tile_y;
@@ -685,14 +693,17 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
             return HYDRO_EUNSUPPORTED;  // the ring's int indices
     }
     const bool rows = grid->dim == 2 && var.tile_y == 1;
-    int strip_rows = 0;
+    int strip_rows = 0, strip_planes = 0;
     if ((grid->dim == 3 || rows) && prec == HYDRO_F32 && !(variant && variant->march)) {
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
             var.march = rows ? default_march_rows(grid->n, var, sms)
                              : default_march_3d(grid->n, var, sms);
-        if (rows) strip_rows = hydro::default_strip_rows(grid->n[0], grid->n[1], sms);
+        if (rows)
+            strip_rows = hydro::default_strip_rows(grid->n[0], grid->n[1], sms);
+        else if (strips3(prec, grid->dim, var))
+            strip_planes = hydro::default_strip_planes(grid->n[0], grid->n[1], grid->n[2], sms);
     }
     const Layout lay = layout_for(grid->dim, grid->n, ncell, prec, var.manifest);
     if (workspace_bytes < lay.total) return HYDRO_EINVAL;
@@ -727,6 +738,8 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
     c->cfl = cfl;
     c->var = var;
     c->strip_rows = strip_rows;
+    c->march = strip_planes ? strip_planes : var.march;
+    if (marching && c->march > c->n[c->dim - 1]) c->march = c->n[c->dim - 1];
     c->lay = lay;
     c->ws = static_cast<unsigned char *>(workspace);
     c->ctrl = reinterpret_cast<Ctrl *>(c->ws + lay.ctrl_off);
@@ -884,7 +897,7 @@ static cudaError_t copy_planes(void *const dst[5], const void *const src[5], int
 // when its stage-2 launch ends: stage 2 writes only its own cells and reads other slabs' U1,
 // not U.  Returns with the copy stream joined into the context's stream.
 static int last_step_overlapped(hydro_ctx *c, const hydro_state_t *s, void *const host_out[5]) {
-    const int march = c->var.march;
+    const int march = c->march;
     const int nchunks = (c->n[2] + march - 1) / march;
     const int nslabs = nchunks < 8 ? nchunks : 8;
     while ((int)c->slab_events.size() < nslabs + 1) {

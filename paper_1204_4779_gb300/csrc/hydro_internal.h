@@ -48,6 +48,10 @@ cudaError_t stage_f64(int dim, const StageLaunch &L, cudaStream_t st, bool prepa
 // The FP32 row tiles of dim 2 (stage_rows.cu), and the rows a warp of theirs marches through by
 // default on an nx x ny grid.
 cudaError_t stage_rows_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only);
+// The FP32 strip kernels of dim 3 (stage_strip3.cu), and the planes a CTA of theirs marches
+// through by default.
+cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only);
+int default_strip_planes(long long nx, long long ny, long long nz, int sm_count);
 int default_strip_rows(long long nx, long long ny, int sm_count);
 
 // Compiled tile shapes (both_pf: both staging depths compiled).

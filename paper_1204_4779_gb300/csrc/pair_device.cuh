@@ -63,19 +63,8 @@ __device__ __forceinline__ void prim_of_cons_pair(const F2 (&u)[D + 2], F2 (&v)[
     v[D + 1] = f2_mul(G.gm1, f2_fma(f2_splat(-0.5f), kin, u[D + 1]));
 }
 
-// HLLC flux of a pair of faces; velocities and flux normal-first, as in hllc().
-//
-// With the wave speeds clamped (S_L to <= 0, S_R to >= 0) the jump condition
-// F* = F_K + S (U* - U_K) covers all four cases: on a supersonic face S is 0 and F* = F_K.
-// Written in the star state it needs neither F_K nor U_K.  With m = r (u - S),
-// p* = p + m (u - S*) and q = S* / (S* - S) (q = 1 where S = 0),
-//     F_mass = m q,  F_normal = F_mass S* + p*,  F_tangential = F_mass v_t,
-//     F_E    = p* S* + q (p ((u - S) / (gamma - 1) + u) + m v^2 / 2 - p* S*).
-// The clamped speeds also enter S*: it is then the same wherever no wave speed has passed zero,
-// and its sign, which chooses the side, is the same everywhere (Davis speeds: if S_R <= 0, both
-// sides' u <= -a, and the numerator of S* is at least (gamma - 1) p_L + (gamma + 1) p_R > 0 with
-// either S_R, so S* < 0).  The pressure-based estimate bounds only its own side's velocity, so
-// there S* comes from the unclamped speeds.
+// HLLC flux of a pair of faces; velocities and flux normal-first.  The operations of the FP32
+// hllc(), on both lanes.
 template <int D>
 __device__ __forceinline__ void hllc_pair(F2 rl, const F2 (&vl)[D], F2 pl, F2 rr,
                                           const F2 (&vr)[D], F2 pr, const PairGas &G,
@@ -104,21 +93,9 @@ __device__ __forceinline__ void hllc_pair(F2 rl, const F2 (&vl)[D], F2 pl, F2 rr
         f2_unpack(ar, c2[0], c2[1]);
         f2_unpack(ul, u1[0], u1[1]);
         f2_unpack(ur, u2[0], u2[1]);
-        const float g = f2_lo(G.g), c = __fmul_rn(__fadd_rn(g, 1.0f), __fmul_rn(0.5f, Arith<float>::rcp(g)));
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const float ra = __fmul_rn(__fmul_rn(0.5f, __fadd_rn(l[i], r[i])),
-                                       __fmul_rn(0.5f, __fadd_rn(c1[i], c2[i])));
-            const float ps = fmaxf(0.0f, fmaf(__fmul_rn(-0.5f, __fadd_rn(u2[i], -u1[i])), ra,
-                                              __fmul_rn(0.5f, __fadd_rn(p1[i], p2[i]))));
-            float ql = 1.0f, qr = 1.0f;
-            if (!(ps <= p1[i]))
-                ql = Arith<float>::sqrt_(fmaf(c, fmaf(ps, Arith<float>::rcp(p1[i]), -1.0f), 1.0f));
-            if (!(ps <= p2[i]))
-                qr = Arith<float>::sqrt_(fmaf(c, fmaf(ps, Arith<float>::rcp(p2[i]), -1.0f), 1.0f));
-            SL[i] = fmaf(-c1[i], ql, u1[i]);
-            SR[i] = fmaf(c2[i], qr, u2[i]);
-        }
+        for (int i = 0; i < 2; ++i)
+            pvrs_speeds(l[i], u1[i], p1[i], c1[i], r[i], u2[i], p2[i], c2[i], f2_lo(G.g), SL[i], SR[i]);
     }
     const F2 ml = f2_mul(rl, f2_sub(f2_pack(SL[0], SL[1]), ul));
     const F2 nr = f2_mul(rr, f2_sub(ur, f2_pack(SR[0], SR[1])));  // -m_R

@@ -174,6 +174,11 @@ template <class T, int NV> struct Pairs {
     static constexpr int first_scalar = 2 * n;
 };
 
+// a + c x: one FMA in FP32 (spelled out, so that every kernel rounds alike), a product and a sum
+// in FP64
+__device__ __forceinline__ float add_scaled(float a, float c, float x) { return fmaf(c, x, a); }
+__device__ __forceinline__ double add_scaled(double a, double c, double x) { return a + c * x; }
+
 // MinBee slopes d = minbee(c - m, p - c) of three consecutive cells, value by value (all zero
 // for first-order reconstruction).
 template <class T, int NV>
@@ -215,8 +220,7 @@ __device__ __forceinline__ void half_step(const T (&v)[NV], const T (&d)[NV], T 
         }
     }
 #pragma unroll
-    for (int k = P::first_scalar; k < NV; ++k)
-        out[k] = (s > T(0)) ? v[k] + T(0.5) * d[k] : v[k] - T(0.5) * d[k];
+    for (int k = P::first_scalar; k < NV; ++k) out[k] = add_scaled(v[k], (s > T(0)) ? T(0.5) : T(-0.5), d[k]);
 }
 
 // MinBee faces of four consecutive cells q0..q3 along a normal: L = upper face of q1,
@@ -243,8 +247,8 @@ __device__ __forceinline__ void minbee_face_pair(const T (&q0)[NV], const T (&q1
 #pragma unroll
     for (int k = P::first_scalar; k < NV; ++k) {
         const T d01 = q1[k] - q0[k], d12 = q2[k] - q1[k], d23 = q3[k] - q2[k];
-        L[k] = q1[k] + T(0.5) * minbee(d01, d12);
-        R[k] = q2[k] - T(0.5) * minbee(d12, d23);
+        L[k] = add_scaled(q1[k], T(0.5), minbee(d01, d12));
+        R[k] = add_scaled(q2[k], T(-0.5), minbee(d12, d23));
     }
 }
 
@@ -273,8 +277,8 @@ __device__ __forceinline__ void add_fluxes(const T (&base)[NV], T cx, const T (&
 #pragma unroll
     for (int k = P::first_scalar; k < NV; ++k) {
         T sum = cx * (fw[k] - fe[k]);
-        if constexpr (HAS_Y) sum = sum + cy * (fs[k] - fn[k]);
-        if constexpr (HAS_M) sum = sum + cz * (zm[k] - zp[k]);
+        if constexpr (HAS_Y) sum = add_scaled(sum, cy, fs[k] - fn[k]);
+        if constexpr (HAS_M) sum = add_scaled(sum, cz, zm[k] - zp[k]);
         un[k] = base[k] + sum;
     }
 }
@@ -309,7 +313,7 @@ __device__ __forceinline__ void inplane_face(const T *__restrict__ sV, T *__rest
         vr[1] = a ? R[1] : R[2];
     }
     if constexpr (D == 3) vl[2] = L[3], vr[2] = R[3];
-    hllc<T, D, false>(L[0], vl, L[NV - 1], R[0], vr, R[NV - 1], G, F, riemann);
+    hllc<D, false>(L[0], vl, L[NV - 1], R[0], vr, R[NV - 1], G, F, riemann);
     T Fa[NV];  // back to axis order
     Fa[0] = F[0];
     Fa[1] = (D >= 2 && a) ? F[2] : F[1];
@@ -334,7 +338,7 @@ __device__ __forceinline__ void march_face(const T (&Vlo)[D + 2], const T (&dlo)
     vr[0] = R[D];
 #pragma unroll
     for (int b = 1; b < D; ++b) vl[b] = L[b], vr[b] = R[b];
-    hllc<T, D, true>(L[0], vl, L[D + 1], R[0], vr, R[D + 1], G, F, riemann);
+    hllc<D, true>(L[0], vl, L[D + 1], R[0], vr, R[D + 1], G, F, riemann);
 }
 
 // Shared-memory position (lx, ly) of halo task h of a BX x BY tile (the cross-shaped two-cell

@@ -1,0 +1,98 @@
+// Launches of the FP32 3D strip kernels (strip3_kernel.cuh).
+#include <math.h>
+
+#include "hydro_internal.h"
+#include "stage_launch.cuh"
+#include "strip3_kernel.cuh"
+
+namespace hydro {
+
+namespace {
+
+template <int SEG, int STAGE, bool CFL> struct Strip3Kernels {
+    // [vectorised][scheme options other than the default]
+    static constexpr void (*k[2][2])(StageArgs<float>) = {
+        {strip3_kernel<SEG, STAGE, CFL, false, false>, strip3_kernel<SEG, STAGE, CFL, false, true>},
+        {strip3_kernel<SEG, STAGE, CFL, true, false>, strip3_kernel<SEG, STAGE, CFL, true, true>}};
+    static cudaError_t prepare() {
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < 4 && e == cudaSuccess; ++i)
+            e = cudaFuncSetAttribute(k[i >> 1][i & 1], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)Strip3<SEG>::bytes);
+        return e;
+    }
+};
+
+template <int SEG> long long strip3_tiles_x(long long nx) {
+    return (nx + Strip3<SEG>::cells - 1) / Strip3<SEG>::cells;
+}
+template <int SEG> long long strip3_tiles_y(long long ny) {
+    return (ny + Strip3<SEG>::NR - 1) / Strip3<SEG>::NR;
+}
+// Rows of 32 lanes unless the grid leaves more columns and rows of theirs unused than of the
+// 16-lane ones: a CTA of either covers 448 cells of a plane.
+bool strip3_half_rows(long long nx, long long ny) {
+    return strip3_tiles_x<16>(nx) * strip3_tiles_y<16>(ny) < strip3_tiles_x<32>(nx) * strip3_tiles_y<32>(ny);
+}
+
+template <int SEG> cudaError_t launch_strip3(const StageLaunch &L, StageArgs<float> &A, cudaStream_t st) {
+    A.tiles_x = (int)strip3_tiles_x<SEG>(A.n[0]);
+    A.tiles_y = (int)strip3_tiles_y<SEG>(A.n[1]);
+    const int chunks = L.zchunks > 0 ? L.zchunks : (A.n[2] + A.march - 1) / A.march - L.zchunk0;
+    const long long ctas = (long long)A.tiles_x * A.tiles_y * chunks;
+    if (ctas < 1 || ctas >= (1LL << 31)) return cudaErrorInvalidValue;
+    const bool vec = rows_vec(L.uin, 5, A.n[0]) && rows_vec(L.ubase, 5, A.n[0]) &&
+                     rows_vec(const_cast<const void *const *>(L.uout), 5, A.n[0]);
+    const bool gen = A.order != 2 || A.riemann != 0;
+    const auto k = L.stage == 1 ? Strip3Kernels<SEG, 1, false>::k[vec][gen]
+                                : (L.split ? Strip3Kernels<SEG, 2, false>::k[vec][gen]
+                                           : Strip3Kernels<SEG, 2, true>::k[vec][gen]);
+    k<<<(unsigned)ctas, kStripThreads, Strip3<SEG>::bytes, st>>>(A);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only) {
+    if (prepare_only) {
+        cudaError_t e = Strip3Kernels<32, 1, false>::prepare();
+        if (e == cudaSuccess) e = Strip3Kernels<32, 2, false>::prepare();
+        if (e == cudaSuccess) e = Strip3Kernels<32, 2, true>::prepare();
+        if (e == cudaSuccess) e = Strip3Kernels<16, 1, false>::prepare();
+        if (e == cudaSuccess) e = Strip3Kernels<16, 2, false>::prepare();
+        return e == cudaSuccess ? Strip3Kernels<16, 2, true>::prepare() : e;
+    }
+    StageArgs<float> A = make_stage_args<float>(L);
+    return strip3_half_rows(A.n[0], A.n[1]) ? launch_strip3<16>(L, A, st)
+                                            : launch_strip3<32>(L, A, st);
+}
+
+// Planes a CTA marches through when the variant names no march: the least (m + 1.5) x waves, a
+// chunk's prologue counted as 1.5 planes, the waves of the resident CTAs (two per SM) counted by
+// work (the last chunk may be short) with the last one whole, or 0.62 where no SM gets a second
+// CTA of it.  Measured on GB300, blast, us per step at m = 4 / 8 / 12 / 16 / 24 / 32 / 64 / 96,
+// chosen marked:
+//   64^3   30.0* 31.3  40.7  49.9  68.5  86.8  161
+//   128^3  119   116   112   114   110*  142   164   241
+//   192^3  327   299   296   286   308   279   276*  402
+//   256^3  792   710   686   680   676   664*  664   707
+//   512^3  5651  5025  4822  4719  4610  4582  4560* 4472
+int default_strip_planes(long long nx, long long ny, long long nz, int sm_count) {
+    static const int kPlanes[] = {2, 4, 6, 8, 12, 16, 20, 24, 32, 40, 48, 64, 80, 96, 128};
+    const double tiles = strip3_half_rows(nx, ny)
+                             ? (double)(strip3_tiles_x<16>(nx) * strip3_tiles_y<16>(ny))
+                             : (double)(strip3_tiles_x<32>(nx) * strip3_tiles_y<32>(ny));
+    const double slots = 2.0 * (sm_count > 0 ? sm_count : 1);
+    int best = 0;
+    double best_cost = 0.0;
+    for (int m : kPlanes) {
+        const double waves =
+            tiles * ((double)nz + 1.5 * (double)((nz + m - 1) / m)) / ((m + 1.5) * slots);
+        const double whole = floor(waves), rest = waves - whole;
+        const double cost = (m + 1.5) * (whole + (rest > 0.5 || whole == 0.0 ? 1.0 : (rest > 0.0 ? 0.62 : 0.0)));
+        if (best == 0 || cost < best_cost) best = m, best_cost = cost;
+    }
+    return best;
+}
+
+}  // namespace hydro
