@@ -47,7 +47,7 @@ UNITS = {
     "exchange.cu": [],
     "tma_host.cu": [],
 }
-HEADERS = ["hydro_device.cuh", "stage_kernel.cuh", "stage_launch.cuh", "hydro_internal.h",
+HEADERS = ["hydro_device.cuh", "exact64.cuh", "stage_kernel.cuh", "stage_launch.cuh", "hydro_internal.h",
            "batch_kernel.cuh", "tma.cuh", "pair_device.cuh", "row_kernel.cuh",
            "strip3_kernel.cuh"]
 

@@ -64,9 +64,7 @@ __global__ void __launch_bounds__(kAuxThreads) cfl_kernel(const AuxT<T> A) {
         prim_of_cons<T, D>(u, v, A.gas);
         T s = T(0);
         if constexpr (Arith<T>::exact) {
-            const T cs = sqrt(A.gas.g * v[NV - 1] / v[0]);
-#pragma unroll
-            for (int a = 0; a < D; ++a) s = s + (fabs(v[1 + a]) + cs) / T(A.dr[a]);
+            s = exact_signal<D>(v, A.gas, A.dr, A.inv_dr);
         } else {
             const T cs = Arith<float>::sqrt_(A.gas.g * v[NV - 1] * Arith<float>::rcp(v[0]));
 #pragma unroll

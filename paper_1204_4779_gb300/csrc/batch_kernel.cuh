@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(BX * BY, (MinBlocks<T, BX * BY>::value))
             Cells<T, NV>::get(sF, NF, fxl + 1, fe);
             Cells<T, NV>::get(sF, NF, fyb, fs);
             Cells<T, NV>::get(sF, NF, fyb + BX, fn);
-            add_fluxes<T, NV, true, false>(base, cx, fw, fe, cy, fs, fn, T(0), fw, fw, un);
+            add_fluxes<T, NV, true, false>(base, cx, fw, fe, cy, fs, fn, T(0), fw, fw, un, G.x);
             const long long i = off + (long long)y * nx + x;
 #pragma unroll
             for (int k = 0; k < NV; ++k) A.uout[k][i] = un[k];

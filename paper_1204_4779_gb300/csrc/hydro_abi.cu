@@ -219,6 +219,26 @@ int default_march_3d(const int64_t n[3], const hydro_variant_t &v, int sm_count)
     return choose_march(tiles, n[2], resident_slots(v, sm_count), 3.0, kMarch, 9, 8);
 }
 
+// Planes a CTA of the FP64 3D tiles marches through when the variant names no march (the reported
+// default stays 64): one CTA of 256 threads fits an SM and keeps its FP64 pipe busy, so a launch
+// takes (m + 0.7) x (CTAs the busiest SM gets), a chunk's prologue (four recoveries, one face of
+// three) counted as 0.7 planes.  97 x 83 x 75 in chunks of 64 made 88 CTAs for 152 SMs.
+int default_march_f64_3d(const int64_t n[3], const hydro_variant_t &v, int sm_count) {
+    const long long tiles = ((n[0] + v.tile_x - 1) / v.tile_x) * ((n[1] + v.tile_y - 1) / v.tile_y);
+    const long long sms = sm_count > 0 ? sm_count : 1;
+    int best = 64;
+    double best_cost = 0.0;
+    for (int m = 1; m <= 64; ++m) {
+        const long long items = tiles * ((n[2] + m - 1) / m);
+        // over many rounds the SMs even out
+        const double rounds = items > 8 * sms ? (double)items / (double)sms + 0.5
+                                              : (double)((items + sms - 1) / sms);
+        const double cost = (m + 0.7) * rounds;
+        if (best_cost == 0.0 || cost <= best_cost) best = m, best_cost = cost;
+    }
+    return best;
+}
+
 // Default march of the 2D FP32 row tiles (a variant that names no march), with the same cost
 // and marches 8, 16, 32, 64, 128 whose items fill the resident CTAs twice (launches of more
 // items than resident CTAs run persistently, so a short last wave costs little); 16 when none
@@ -310,8 +330,8 @@ struct hydro_ctx {
     void *frame[5] = {};
     hydro_variant_t var = {};
     int strip_rows = 0;      // FP32 row tiles without a named march: rows of a warp
-    int march = 1;           // planes of a chunk: the variant's, or where it names none and the
-                             // 3D strip kernels run, their own choice
+    int march = 1;           // planes of a chunk: the variant's, or where it names none the
+                             // choice of the 3D strip kernels or of the FP64 tiles
     Layout lay = {};
     unsigned char *ws = nullptr;
     Ctrl *ctrl = nullptr;
@@ -693,7 +713,13 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
             return HYDRO_EUNSUPPORTED;  // the ring's int indices
     }
     const bool rows = grid->dim == 2 && var.tile_y == 1;
-    int strip_rows = 0, strip_planes = 0;
+    int strip_rows = 0, own_march = 0;
+    if (grid->dim == 3 && prec == HYDRO_F64 && !(variant && variant->march)) {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+            own_march = default_march_f64_3d(grid->n, var, sms);
+    }
     if ((grid->dim == 3 || rows) && prec == HYDRO_F32 && !(variant && variant->march)) {
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -703,7 +729,7 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
         if (rows)
             strip_rows = hydro::default_strip_rows(grid->n[0], grid->n[1], sms);
         else if (strips3(prec, grid->dim, var))
-            strip_planes = hydro::default_strip_planes(grid->n[0], grid->n[1], grid->n[2], sms);
+            own_march = hydro::default_strip_planes(grid->n[0], grid->n[1], grid->n[2], sms);
     }
     const Layout lay = layout_for(grid->dim, grid->n, ncell, prec, var.manifest);
     if (workspace_bytes < lay.total) return HYDRO_EINVAL;
@@ -738,7 +764,7 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
     c->cfl = cfl;
     c->var = var;
     c->strip_rows = strip_rows;
-    c->march = strip_planes ? strip_planes : var.march;
+    c->march = own_march ? own_march : var.march;
     if (marching && c->march > c->n[c->dim - 1]) c->march = c->n[c->dim - 1];
     c->lay = lay;
     c->ws = static_cast<unsigned char *>(workspace);

@@ -15,6 +15,8 @@
 
 #include <type_traits>
 
+#include "exact64.cuh"
+
 namespace hydro {
 
 // ----------------------------------------------------------------- control block ----------
@@ -148,7 +150,8 @@ __device__ __forceinline__ void acc_add(DF &s, DF x) {
 template <class T> struct Gas {
     T g;        // gamma
     T gm1;      // gamma - 1
-    T inv_gm1;  // 1 / (gamma - 1)  (FP32 mode only)
+    T inv_gm1;  // 1 / (gamma - 1)
+    Fma64 x;    // FP64 mode's constants
 };
 
 template <class T> __host__ __device__ inline Gas<T> make_gas(double gamma) {
@@ -156,8 +159,15 @@ template <class T> __host__ __device__ inline Gas<T> make_gas(double gamma) {
     G.g = T(gamma);
     G.gm1 = T(gamma - 1.0);
     G.inv_gm1 = T(1.0 / (gamma - 1.0));
+    G.x.one = 1.0;
+    G.x.mzero = -0.0;
     return G;
 }
+
+// FP64 operations for operands the arithmetic of exact64.cuh leaves out, out of line (scalars
+// only: the callers' arrays stay in registers).
+static __device__ __noinline__ double div_plain(double a, double b) { return a / b; }
+static __device__ __noinline__ double root_plain(double a) { return sqrt(a); }
 
 // V(U) for one cell: v_a = m_a / rho, p = (gamma - 1)(E - rho v^2 / 2), the kinetic term
 // summed in axis order as m_a v_a.
@@ -166,13 +176,27 @@ __device__ __forceinline__ void prim_of_cons(const T (&u)[D + 2], T (&v)[D + 2],
     const T rho = u[0];
     v[0] = rho;
     if constexpr (Arith<T>::exact) {
+        // the plain form's values (0.5 kin is exact, so the FMA rounds once, as the difference)
+        bool ok = in_range(rho) && positive(rho);
+        const T y = recip64(rho);
         T kin = T(0);
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-            v[1 + a] = u[1 + a] / rho;
-            kin = kin + u[1 + a] * v[1 + a];
+            ok &= in_range(u[1 + a]) || is_zero(u[1 + a]);
+            v[1 + a] = G.x.div(u[1 + a], rho, y);
+            const T e = G.x.mul(u[1 + a], v[1 + a]);
+            kin = a == 0 ? e : G.x.add(kin, e);
         }
-        v[D + 1] = G.gm1 * (u[D + 1] - T(0.5) * kin);
+        v[D + 1] = G.x.mul(G.gm1, fma(-0.5, kin, u[D + 1]));
+        if (!ok) {
+            kin = T(0);
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+                v[1 + a] = div_plain(u[1 + a], rho);
+                kin = kin + u[1 + a] * v[1 + a];
+            }
+            v[D + 1] = G.gm1 * (u[D + 1] - T(0.5) * kin);
+        }
     } else {
         const T ir = Arith<float>::rcp(rho);
         T kin = T(0);
@@ -187,8 +211,17 @@ __device__ __forceinline__ void prim_of_cons(const T (&u)[D + 2], T (&v)[D + 2],
 
 // MinBee slope of Eq. eqInterpolateSingle from the two one-sided differences:
 // 0 if d01 d12 < 0, else the one of smaller magnitude (d12 on a tie).
+// FP64 on the bit patterns.  d01 d12 < 0: the signs differ, neither is zero or NaN, and the
+// product does not underflow (differences that small are multiplied out).
 __device__ __forceinline__ double minbee(double d01, double d12) {
-    return (d01 * d12 < 0.0) ? 0.0 : (fabs(d01) < fabs(d12) ? d01 : d12);
+    const unsigned long long a = (unsigned long long)__double_as_longlong(d01) & 0x7fffffffffffffffull;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d12) & 0x7fffffffffffffffull;
+    const int ah = (int)(a >> 32), bh = (int)(b >> 32);
+    constexpr int kNan = 0x7ff80000;
+    bool opposite = (__double2hiint(d01) ^ __double2hiint(d12)) < 0 && a != 0ull && b != 0ull &&
+                    max(ah, bh) < kNan;
+    if (opposite && (ah >> 20) + (bh >> 20) < 1100) opposite = d01 * d12 < 0.0;
+    return opposite ? 0.0 : (a < b && bh < kNan ? d01 : d12);
 }
 // FP32 form in three ALU operations: min.xorsign.abs gives min(|a|, |b|) carrying a negative
 // sign exactly when the signs of a and b differ; clamping at zero yields 0 for opposite signs;
@@ -211,15 +244,16 @@ __device__ __forceinline__ float minbee(float d01, float d12) {
 // shock, S_L = u_L - a_L q_L, S_R = u_R + a_R q_R).
 //
 // FP64: F_L if S_L >= 0; F*_L if S* >= 0; F*_R if S_R > 0; else F_R, with the formulas' own
-// operations in their order.
+// operations in their order.  The plain form, for operands the fast one below leaves out and
+// the pressure-based speeds.
 template <int D, bool NLAST>
-__device__ __forceinline__ void hllc(double rl, const double (&vl)[D], double pl, double rr,
-                                     const double (&vr)[D], double pr, const Gas<double> &G,
-                                     double (&F)[D + 2], int riemann = 0) {
+__device__ __forceinline__ void hllc_plain(double rl, const double (&vl)[D], double pl, double rr,
+                                           const double (&vr)[D], double pr, const Gas<double> &G,
+                                           double (&F)[D + 2], int riemann) {
     using T = double;
     const T ul = vl[0], ur = vr[0];
-    const T al = sqrt(G.g * pl / rl);
-    const T ar = sqrt(G.g * pr / rr);
+    const T al = root_plain(div_plain(G.g * pl, rl));
+    const T ar = root_plain(div_plain(G.g * pr, rr));
     T SL, SR;
     if (riemann == 0) {
         SL = fmin(ul - al, ur - ar);
@@ -230,15 +264,15 @@ __device__ __forceinline__ void hllc(double rl, const double (&vl)[D], double pl
         const T ppv = T(0.5) * (pl + pr) - T(0.5) * (ur - ul) * rbar * abar;
         const T ps = fmax(T(0), ppv);
         T ql = T(1), qr = T(1);
-        const T c = (G.g + T(1)) / (T(2) * G.g);
-        if (!(ps <= pl)) ql = sqrt(T(1) + c * (ps / pl - T(1)));
-        if (!(ps <= pr)) qr = sqrt(T(1) + c * (ps / pr - T(1)));
+        const T c = div_plain(G.g + T(1), T(2) * G.g);
+        if (!(ps <= pl)) ql = root_plain(T(1) + c * (div_plain(ps, pl) - T(1)));
+        if (!(ps <= pr)) qr = root_plain(T(1) + c * (div_plain(ps, pr) - T(1)));
         SL = ul - al * ql;
         SR = ur + ar * qr;
     }
     const T ml = rl * (SL - ul);
     const T mr = rr * (SR - ur);
-    const T Ss = (pr - pl + rl * ul * (SL - ul) - rr * ur * (SR - ur)) / (ml - mr);
+    const T Ss = div_plain(pr - pl + rl * ul * (SL - ul) - rr * ur * (SR - ur), ml - mr);
 
     const bool left = (T(0) <= SL) || (T(0) <= Ss);
     const bool star = !(T(0) <= SL) && ((T(0) <= Ss) || (T(0) < SR));
@@ -266,15 +300,15 @@ __device__ __forceinline__ void hllc(double rl, const double (&vl)[D], double pl
     FK[0] = r * u;
 #pragma unroll
     for (int b = 0; b < D; ++b) U[1 + b] = r * v[b];
-    U[D + 1] = p / G.gm1 + T(0.5) * r * v2;
+    U[D + 1] = div_plain(p, G.gm1) + T(0.5) * r * v2;
     FK[1] = U[1] * u + p;
 #pragma unroll
     for (int b = 1; b < D; ++b) FK[1 + b] = U[1 + b] * u;
     FK[D + 1] = u * (U[D + 1] + p);
 
     // star state: rho (S - u)/(S - S*) (1, S*, v_t, E/rho + (S* - u)(S* + p/(rho (S - u))))
-    const T chi = r * (S - u) / (S - Ss);
-    const T eterm = U[D + 1] / r + (Ss - u) * (Ss + p / (r * (S - u)));
+    const T chi = div_plain(r * (S - u), S - Ss);
+    const T eterm = div_plain(U[D + 1], r) + (Ss - u) * (Ss + div_plain(p, r * (S - u)));
     T Us[D + 2];
     Us[0] = chi;
     Us[1] = chi * Ss;
@@ -283,6 +317,81 @@ __device__ __forceinline__ void hllc(double rl, const double (&vl)[D], double pl
     Us[D + 1] = chi * eterm;
 #pragma unroll
     for (int k = 0; k < D + 2; ++k) F[k] = star ? FK[k] + S * (Us[k] - U[k]) : FK[k];
+}
+
+// The same values by the arithmetic of exact64.cuh: about 105 FP64 operations a face in 3D
+// where the plain form issues 150.  5 reciprocals serve 7 quotients; S - u, r (S - u) and r u of
+// the chosen side are selected, not computed again; 0.5 r v^2 is added by an FMA (the half is
+// exact).
+template <int D, bool NLAST>
+__device__ __forceinline__ void hllc(double rl, const double (&vl)[D], double pl, double rr,
+                                     const double (&vr)[D], double pr, const Gas<double> &G,
+                                     double (&F)[D + 2], int riemann = 0) {
+    const Fma64 &X = G.x;
+    const double ul = vl[0], ur = vr[0];
+    bool ok = riemann == 0 && in_range(rl) && in_range(rr) && in_range(pl) && in_range(pr) &&
+              positive(rl) && positive(rr) && positive(pl) && positive(pr);
+    const double yl = recip64(rl), yr = recip64(rr);
+    const double al = sqrt64(X.div(X.mul(G.g, pl), rl, yl), X);
+    const double ar = sqrt64(X.div(X.mul(G.g, pr), rr, yr), X);
+    const double la = X.sub(ul, al), lb = X.sub(ur, ar), ra = X.add(ul, al), rb = X.add(ur, ar);
+    const double SL = less(lb, la) ? lb : la, SR = less(ra, rb) ? rb : ra;
+    const double sl = X.sub(SL, ul), sr = X.sub(SR, ur);
+    const double ml = X.mul(rl, sl), mr = X.mul(rr, sr);
+    const double rul = X.mul(rl, ul), rur = X.mul(rr, ur);
+    const double num = X.sub(X.add(X.sub(pr, pl), X.mul(rul, sl)), X.mul(rur, sr));
+    const double den = X.sub(ml, mr);
+    ok = ok && in_range(den) && (in_range(num) || is_zero(num));
+    const double Ss = X.div(num, den, recip64(den));
+    const bool left = ge0(SL) || ge0(Ss);
+    const bool star = !ge0(SL) && (ge0(Ss) || gt0(SR));
+    const double r = left ? rl : rr, p = left ? pl : pr, S = left ? SL : SR;
+    const double y = left ? yl : yr, m = left ? ml : mr;
+    double v[D];
+#pragma unroll
+    for (int b = 0; b < D; ++b) v[b] = left ? vl[b] : vr[b];
+    const double u = v[0];
+    // v^2 in axis order
+    double v2;
+    if constexpr (NLAST && D > 1) {
+        v2 = X.mul(v[1], v[1]);
+#pragma unroll
+        for (int b = 2; b < D; ++b) v2 = X.add(v2, X.mul(v[b], v[b]));
+        v2 = X.add(v2, X.mul(u, u));
+    } else {
+        v2 = X.mul(u, u);
+#pragma unroll
+        for (int b = 1; b < D; ++b) v2 = X.add(v2, X.mul(v[b], v[b]));
+    }
+    double U[D + 2], FK[D + 2];
+    U[0] = r;
+    U[1] = left ? rul : rur;
+    FK[0] = U[1];
+#pragma unroll
+    for (int b = 1; b < D; ++b) U[1 + b] = X.mul(r, v[b]);
+    const double E = fma(0.5, X.mul(r, v2), X.div(p, G.gm1, G.inv_gm1));
+    U[D + 1] = E;
+    FK[1] = X.add(X.mul(U[1], u), p);
+#pragma unroll
+    for (int b = 1; b < D; ++b) FK[1 + b] = X.mul(U[1 + b], u);
+    FK[D + 1] = X.mul(u, X.add(E, p));
+    const double sd = X.sub(S, Ss);
+    ok = ok && in_range(E) && (!star || (in_range(sd) && in_range(m)));
+    const double chi = X.div(m, sd, recip64(sd));
+    const double eterm = X.add(X.div(E, r, y),
+                               X.mul(X.sub(Ss, u), X.add(Ss, X.div(p, m, recip64(m)))));
+    double Us[D + 2];
+    Us[0] = chi;
+    Us[1] = X.mul(chi, Ss);
+#pragma unroll
+    for (int b = 1; b < D; ++b) Us[1 + b] = X.mul(chi, v[b]);
+    Us[D + 1] = X.mul(chi, eterm);
+#pragma unroll
+    for (int k = 0; k < D + 2; ++k) {
+        const double f = X.add(FK[k], X.mul(S, X.sub(Us[k], U[k])));
+        F[k] = star ? f : FK[k];
+    }
+    if (!ok) hllc_plain<D, NLAST>(rl, vl, pl, rr, vr, pr, G, F, riemann);
 }
 
 // Pressure-based wave speeds of one face in FP32, every operation named by its rounding.
@@ -354,6 +463,30 @@ __device__ __forceinline__ void hllc(float rl, const float (&vl)[D], float pl, f
     const float x = __fmul_rn(ps, Ss);
     const float t = fmaf(__fmul_rn(0.5f, m), v2, __fmul_rn(p, fmaf(us, G.inv_gm1, u)));
     F[D + 1] = fmaf(q, __fadd_rn(t, -x), x);
+}
+
+// CFL signal sum_a (|v_a| + c_s) / dr_a of an FP64 primitive state, c_s = sqrt(gamma p / rho).
+template <int D>
+__device__ __forceinline__ double exact_signal(const double (&v)[D + 2], const Gas<double> &G,
+                                               const double *dr, const double *inv_dr) {
+    const Fma64 &X = G.x;
+    bool ok = in_range(v[0]) && in_range(v[D + 1]) && positive(v[0]) && positive(v[D + 1]);
+    const double cs = sqrt64(X.div(X.mul(G.g, v[D + 1]), v[0], recip64(v[0])), X);
+    double s = 0.0;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        const double w = X.add(fabs(v[1 + a]), cs);
+        ok = ok && in_range(w) && in_range(dr[a]);
+        const double q = X.div(w, dr[a], inv_dr[a]);
+        s = a == 0 ? q : X.add(s, q);
+    }
+    if (!ok) {
+        const double c = root_plain(div_plain(G.g * v[D + 1], v[0]));
+        s = 0.0;
+#pragma unroll
+        for (int a = 0; a < D; ++a) s = s + div_plain(fabs(v[1 + a]) + c, dr[a]);
+    }
+    return s;
 }
 
 // Boundary remap of a cell index at most two cells outside [0, n): periodic wraps once,

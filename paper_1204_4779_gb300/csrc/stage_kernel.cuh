@@ -76,11 +76,10 @@ __device__ __forceinline__ void cfl_signal(const T (&un)[D + 2], const StageArgs
     constexpr int NV = D + 2;
     T v[NV];
     prim_of_cons<T, D>(un, v, A.gas);
-    T cs, s = T(0);
+    [[maybe_unused]] T cs;
+    T s = T(0);
     if constexpr (Arith<T>::exact) {
-        cs = sqrt(A.gas.g * v[NV - 1] / v[0]);
-#pragma unroll
-        for (int a = 0; a < D; ++a) s = s + (fabs(v[1 + a]) + cs) / A.dr[a];
+        s = exact_signal<D>(v, A.gas, A.dr, A.inv_dr);
     } else {
         cs = Arith<float>::sqrt_(A.gas.g * v[NV - 1] * Arith<float>::rcp(v[0]));
 #pragma unroll
@@ -174,16 +173,28 @@ template <class T, int NV> struct Pairs {
     static constexpr int first_scalar = 2 * n;
 };
 
+// FP64 sums, differences and products as fused multiply-adds (exact64.cuh)
+__device__ __forceinline__ float sub_(float a, float b, const Fma64 &) { return a - b; }
+__device__ __forceinline__ double sub_(double a, double b, const Fma64 &X) { return X.sub(a, b); }
+__device__ __forceinline__ float add_(float a, float b, const Fma64 &) { return a + b; }
+__device__ __forceinline__ double add_(double a, double b, const Fma64 &X) { return X.add(a, b); }
+__device__ __forceinline__ float mul_(float a, float b, const Fma64 &) { return a * b; }
+__device__ __forceinline__ double mul_(double a, double b, const Fma64 &X) { return X.mul(a, b); }
 // a + c x: one FMA in FP32 (spelled out, so that every kernel rounds alike), a product and a sum
 // in FP64
-__device__ __forceinline__ float add_scaled(float a, float c, float x) { return fmaf(c, x, a); }
-__device__ __forceinline__ double add_scaled(double a, double c, double x) { return a + c * x; }
+__device__ __forceinline__ float add_scaled(float a, float c, float x, const Fma64 &) { return fmaf(c, x, a); }
+__device__ __forceinline__ double add_scaled(double a, double c, double x, const Fma64 &X) {
+    return X.add(a, X.mul(c, x));
+}
+// a + x / 2 or a - x / 2 (the half is exact, so one FMA rounds as the sum does)
+__device__ __forceinline__ float add_half(float a, float c, float x) { return fmaf(c, x, a); }
+__device__ __forceinline__ double add_half(double a, double c, double x) { return fma(c, x, a); }
 
 // MinBee slopes d = minbee(c - m, p - c) of three consecutive cells, value by value (all zero
 // for first-order reconstruction).
 template <class T, int NV>
 __device__ __forceinline__ void minbee_slopes(const T (&m)[NV], const T (&c)[NV], const T (&p)[NV],
-                                              bool order2, T (&d)[NV]) {
+                                              bool order2, T (&d)[NV], const Fma64 &X) {
     using P = Pairs<T, NV>;
     if (!order2) {
 #pragma unroll
@@ -203,7 +214,7 @@ __device__ __forceinline__ void minbee_slopes(const T (&m)[NV], const T (&c)[NV]
         }
     }
 #pragma unroll
-    for (int k = P::first_scalar; k < NV; ++k) d[k] = minbee(c[k] - m[k], p[k] - c[k]);
+    for (int k = P::first_scalar; k < NV; ++k) d[k] = minbee(sub_(c[k], m[k], X), sub_(p[k], c[k], X));
 }
 
 // Face states from cell values and slopes: out = v + s * d / 2 (s = +1: the cell's upper face,
@@ -220,7 +231,7 @@ __device__ __forceinline__ void half_step(const T (&v)[NV], const T (&d)[NV], T 
         }
     }
 #pragma unroll
-    for (int k = P::first_scalar; k < NV; ++k) out[k] = add_scaled(v[k], (s > T(0)) ? T(0.5) : T(-0.5), d[k]);
+    for (int k = P::first_scalar; k < NV; ++k) out[k] = add_half(v[k], (s > T(0)) ? T(0.5) : T(-0.5), d[k]);
 }
 
 // MinBee faces of four consecutive cells q0..q3 along a normal: L = upper face of q1,
@@ -228,7 +239,7 @@ __device__ __forceinline__ void half_step(const T (&v)[NV], const T (&d)[NV], T 
 template <class T, int NV>
 __device__ __forceinline__ void minbee_face_pair(const T (&q0)[NV], const T (&q1)[NV],
                                                  const T (&q2)[NV], const T (&q3)[NV], T (&L)[NV],
-                                                 T (&R)[NV]) {
+                                                 T (&R)[NV], const Fma64 &X) {
     using P = Pairs<T, NV>;
     if constexpr (P::n > 0) {
         const F2 h = f2_pack(0.5f, 0.5f), mh = f2_pack(-0.5f, -0.5f);
@@ -246,9 +257,9 @@ __device__ __forceinline__ void minbee_face_pair(const T (&q0)[NV], const T (&q1
     }
 #pragma unroll
     for (int k = P::first_scalar; k < NV; ++k) {
-        const T d01 = q1[k] - q0[k], d12 = q2[k] - q1[k], d23 = q3[k] - q2[k];
-        L[k] = add_scaled(q1[k], T(0.5), minbee(d01, d12));
-        R[k] = add_scaled(q2[k], T(-0.5), minbee(d12, d23));
+        const T d01 = sub_(q1[k], q0[k], X), d12 = sub_(q2[k], q1[k], X), d23 = sub_(q3[k], q2[k], X);
+        L[k] = add_half(q1[k], T(0.5), minbee(d01, d12));
+        R[k] = add_half(q2[k], T(-0.5), minbee(d12, d23));
     }
 }
 
@@ -260,7 +271,7 @@ template <class T, int NV, bool HAS_Y, bool HAS_M>
 __device__ __forceinline__ void add_fluxes(const T (&base)[NV], T cx, const T (&fw)[NV],
                                            const T (&fe)[NV], T cy, const T (&fs)[NV],
                                            const T (&fn)[NV], T cz, const T (&zm)[NV],
-                                           const T (&zp)[NV], T (&un)[NV]) {
+                                           const T (&zp)[NV], T (&un)[NV], const Fma64 &X) {
     using P = Pairs<T, NV>;
     if constexpr (P::n > 0) {
         const F2 CX = f2_pack(cx, cx), CY = f2_pack(cy, cy), CZ = f2_pack(cz, cz);
@@ -276,10 +287,10 @@ __device__ __forceinline__ void add_fluxes(const T (&base)[NV], T cx, const T (&
     }
 #pragma unroll
     for (int k = P::first_scalar; k < NV; ++k) {
-        T sum = cx * (fw[k] - fe[k]);
-        if constexpr (HAS_Y) sum = add_scaled(sum, cy, fs[k] - fn[k]);
-        if constexpr (HAS_M) sum = add_scaled(sum, cz, zm[k] - zp[k]);
-        un[k] = base[k] + sum;
+        T sum = mul_(cx, sub_(fw[k], fe[k], X), X);
+        if constexpr (HAS_Y) sum = add_scaled(sum, cy, sub_(fs[k], fn[k], X), X);
+        if constexpr (HAS_M) sum = add_scaled(sum, cz, sub_(zm[k], zp[k], X), X);
+        un[k] = add_(base[k], sum, X);
     }
 }
 
@@ -299,7 +310,7 @@ __device__ __forceinline__ void inplane_face(const T *__restrict__ sV, T *__rest
         T q0[NV], q3[NV];
         C::get(sV, PL, o, q0);
         C::get(sV, PL, o + 3 * s, q3);
-        minbee_face_pair<T, NV>(q0, q1, q2, q3, L, R);
+        minbee_face_pair<T, NV>(q0, q1, q2, q3, L, R, G.x);
     } else {
 #pragma unroll
         for (int k = 0; k < NV; ++k) L[k] = q1[k], R[k] = q2[k];
@@ -601,8 +612,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int x0, int y0
         recover(u, Vc);
         load_u(u, remap(zb + 1, nz, pz), own_off);
         recover(u, Vn);
-        minbee_slopes<T, NV>(Vm2, Vm1, Vc, order2, dzm);
-        minbee_slopes<T, NV>(Vm1, Vc, Vn, order2, dzc);
+        minbee_slopes<T, NV>(Vm2, Vm1, Vc, order2, dzm, G.x);
+        minbee_slopes<T, NV>(Vm1, Vc, Vn, order2, dzc, G.x);
         march_face<T, D>(Vm1, dzm, Vc, dzc, G, Fzm, A.riemann);
         if constexpr (PF == 1) load_u(pown, remap(zb + 2, nz, pz), own_off);
     } else {
@@ -665,7 +676,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int x0, int y0
                 }
                 recover(u, Vnn);
             }
-            minbee_slopes<T, NV>(Vc, Vn, Vnn, order2, dzn);
+            minbee_slopes<T, NV>(Vc, Vn, Vnn, order2, dzn, G.x);
             march_face<T, D>(Vc, dzc, Vn, dzn, G, Fzp, A.riemann);
             // stage plane z+1 into the other buffer, prefetch the halo of plane z+2
             if (z + 1 < ze) {
@@ -739,7 +750,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T> &A, int x0, int y0
                     if (z == nz - 1) A.flux[2][k][iz + (long long)nx * ny] = zp[k];
                 }
             } else {
-                add_fluxes<T, NV, (IN >= 2), MARCH>(base, cx, fw, fe, cy, fs, fn, cz, zm, zp, un);
+                add_fluxes<T, NV, (IN >= 2), MARCH>(base, cx, fw, fe, cy, fs, fn, cz, zm, zp, un, A.gas.x);
                 const int i = (MARCH ? z * pstride : 0) + y * nx + x;
 #pragma unroll
                 for (int k = 0; k < NV; ++k) A.uout[k][i] = un[k];
@@ -919,7 +930,7 @@ __global__ void __launch_bounds__(kPassThreads) addflux_kernel(const StageArgs<T
             zm[k] = A.flux[2][k][i];
             zp[k] = A.flux[2][k][i + plane];
         }
-        add_fluxes<T, NV, true, true>(base, cx, fw, fe, cy, fs, fn, cz, zm, zp, un);
+        add_fluxes<T, NV, true, true>(base, cx, fw, fe, cy, fs, fn, cz, zm, zp, un, A.gas.x);
 #pragma unroll
         for (int k = 0; k < NV; ++k) A.uout[k][i] = un[k];
         if constexpr (STAGE == 2 && FUSED) cfl_signal<T, D>(un, A, smax, bad);
