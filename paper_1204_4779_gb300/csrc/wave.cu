@@ -12,6 +12,10 @@
 // arrays and two workspace arrays.  The translation unit is compiled with --fmad=false: every
 // product and sum of the update formulas is its own IEEE operation, in the formulas' order.
 //
+// Up to kClusterCells cells the whole run is one launch of one thread-block cluster
+// (wave_cluster_kernel): the cells stay in registers, a step costs one cluster barrier.  Larger
+// grids launch per step:
+//
 // FP64, n even and arrays 16-byte aligned (wave_step_kernel_f64v): two cells per thread with
 // 128-bit loads and stores, the neighbours' f1 from the adjacent lanes by warp shuffles; the
 // energy as K1 sum D^2 + K2 sum G^2 (below), each thread's two sums kept in FP64 by fused
@@ -258,6 +262,127 @@ __global__ void __launch_bounds__(kWaveThreads)
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
 
+// All steps of a small grid in one launch of one cluster.  CTA `rank` of C owns cells
+// [rank per, rank per + per); thread t its cells t, t + blockDim.x, ... in registers.  Per step the
+// threads put f1 of their cells into shared memory (the end cells also into the neighbour CTAs'
+// halo slots), meet at one cluster barrier (two buffers alternate), and update g from the
+// neighbours' f1; the update's operations are those of the per-step kernels in their order, so
+// the states are identical.  Each thread's energy term of the step goes to shared memory and one
+// warp, another one each step, adds the CTA's terms in a fixed order after the next barrier: one
+// chain of adds a step instead of one in every warp.
+//
+// Bound by the latency of a step (FP64: 13 operations of 64 cycles for each of a scheduler's
+// warps, the sum's 13 more, the barrier).  N = 3072 FP64: 10.7 us a step by two launches.
+constexpr int kClusterMax = 16;        // CTAs of the cluster (beyond the portable 8)
+constexpr int kClusterThreads = 256;
+constexpr int kClusterPer = 4;         // cells of a thread at most
+constexpr int kClusterCells = kClusterMax * kClusterThreads * kClusterPer;
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Store to a shared variable of CTA `rank` of the cluster (its address in this CTA: a).
+template <class T> __device__ __forceinline__ void store_remote(uint32_t a, unsigned rank, T v) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    if constexpr (sizeof(T) == 4)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
+    else
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+
+// The energy term of one cell, K1 D^2 + K2 G^2.
+__device__ __forceinline__ double wave_term(double fm, double fp, double g0, double g1, double k1,
+                                            double k2) {
+    const double d = fp - fm, s = g0 + g1;
+    return fma(k1 * d, d, k2 * s * s);
+}
+__device__ __forceinline__ double wave_term(float fm, float fp, float g0, float g1, double k1,
+                                            double k2) {
+    const DF d = square(two_sum(fp, -fm)), s = square(two_sum(g0, g1));
+    return k1 * ((double)d.hi + (double)d.lo) + k2 * ((double)s.hi + (double)s.lo);
+}
+
+template <class T>
+__global__ void __launch_bounds__(kClusterThreads)
+    wave_cluster_kernel(T *f, T *g, int n, int per, int n_steps, T dt, T k, double k1, double k2,
+                        double *part) {
+    __shared__ T s_f1[2][kClusterThreads * kClusterPer + 2];
+    __shared__ double s_e[2][kClusterThreads];
+    const int C = gridDim.x, rank = blockIdx.x;
+    const int tid = threadIdx.x, NT = blockDim.x, warps = NT >> 5;
+    const int c0 = rank * per, mine = min(per, n - c0);  // the last CTA may own fewer
+    const int left = rank == 0 ? C - 1 : rank - 1, right = rank == C - 1 ? 0 : rank + 1;
+    const int left_mine = min(per, n - left * per);
+    const uint32_t buf0 = (uint32_t)__cvta_generic_to_shared(&s_f1[0][0]);
+    T fr[kClusterPer], gr[kClusterPer];
+#pragma unroll
+    for (int q = 0; q < kClusterPer; ++q) {
+        const int c = tid + q * NT;
+        fr[q] = c < mine ? f[c0 + c] : T(0);
+        gr[q] = c < mine ? g[c0 + c] : T(0);
+    }
+    // the sum of step s's terms, by warp s % warps, in a fixed order
+    auto reduce = [&](int s) {
+        if ((tid >> 5) != s % warps) return;
+        const double *e = s_e[s & 1];
+        double a = 0.0;
+        for (int i = tid & 31; i < NT; i += 32) a += e[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if ((tid & 31) == 0) part[(long long)s * C + rank] = a;
+    };
+    cluster_sync();  // every CTA of the cluster runs before any writes to its shared memory
+    for (int s = 0; s < n_steps; ++s) {
+        T *const row = s_f1[s & 1];
+        const uint32_t buf = buf0 + (uint32_t)((s & 1) * sizeof(s_f1[0]));
+#pragma unroll
+        for (int q = 0; q < kClusterPer; ++q) {
+            const int c = tid + q * NT;
+            if (c < mine) {
+                fr[q] = fr[q] + dt * gr[q];
+                row[c + 1] = fr[q];
+                if (c == 0) store_remote(buf + (uint32_t)((left_mine + 1) * sizeof(T)), left, fr[q]);
+                if (c == mine - 1) store_remote(buf, right, fr[q]);
+            }
+        }
+        cluster_sync();
+        double e = 0.0;
+#pragma unroll
+        for (int q = 0; q < kClusterPer; ++q) {
+            const int c = tid + q * NT;
+            if (c < mine) {
+                const T fm = row[c], fp = row[c + 2];
+                const T g1 = gr[q] + k * (fp + fm - T(2) * fr[q]);
+                const double t = wave_term(fm, fp, gr[q], g1, k1, k2);
+                e = q == 0 ? t : e + t;
+                gr[q] = g1;
+            }
+        }
+        s_e[s & 1][tid] = e;
+        if (s > 0) reduce(s - 1);  // its terms were written before this step's barrier
+    }
+    __syncthreads();
+    if (n_steps > 0) reduce(n_steps - 1);
+#pragma unroll
+    for (int q = 0; q < kClusterPer; ++q) {
+        const int c = tid + q * NT;
+        if (c < mine) {
+            f[c0 + c] = fr[q];
+            g[c0 + c] = gr[q];
+        }
+    }
+}
+
+// energy[s] = the CTAs' sums of step s in rank order
+__global__ void wave_cluster_energy_kernel(const double *part, int C, int n_steps, double *energy) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n_steps) return;
+    double a = part[(long long)s * C];
+    for (int c = 1; c < C; ++c) a += part[(long long)s * C + c];
+    energy[s] = a;
+}
+
 __global__ void __launch_bounds__(kWaveThreads)
     wave_energy_kernel(const double *partial, int nparts, double *out) {
     __shared__ double s[kWaveThreads];
@@ -290,9 +415,44 @@ WaveLayout wave_layout(long long n, int prec, int n_steps) {
     L.f_off = 0;
     L.g_off = align_up((size_t)n * esz);
     L.part_off = L.g_off + align_up((size_t)n * esz);
-    L.e_off = L.part_off + align_up(sizeof(double) * (size_t)L.nblocks);
+    size_t parts = (size_t)L.nblocks;
+    if (n <= kClusterCells && (size_t)n_steps * kClusterMax > parts)
+        parts = (size_t)n_steps * kClusterMax;  // a sum per CTA of the cluster and step
+    L.e_off = L.part_off + align_up(sizeof(double) * parts);
     L.total = L.e_off + align_up(sizeof(double) * (size_t)(n_steps > 0 ? n_steps : 1));
     return L;
+}
+
+// CTAs of the cluster for n cells: at most one per 64 cells, a power of two, and as many as the
+// device runs at once.
+template <class T> cudaError_t cluster_config(long long n, cudaLaunchConfig_t *cfg,
+                                              cudaLaunchAttribute *attr, cudaStream_t st) {
+    int C = 1;
+    while (C < kClusterMax && n >= 64LL * 2 * C) C *= 2;
+    const auto kernel = wave_cluster_kernel<T>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    for (;;) {
+        const long long per = (n + C - 1) / C;
+        long long threads = (per + 31) / 32 * 32;
+        if (threads > kClusterThreads) threads = kClusterThreads;
+        if (per > threads * kClusterPer) return cudaErrorInvalidValue;
+        attr->id = cudaLaunchAttributeClusterDimension;
+        attr->val.clusterDim.x = (unsigned)C;
+        attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+        cfg->gridDim = dim3((unsigned)C);
+        cfg->blockDim = dim3((unsigned)threads);
+        cfg->dynamicSmemBytes = 0;
+        cfg->stream = st;
+        cfg->attrs = attr;
+        cfg->numAttrs = 1;
+        int fit = 0;
+        e = cudaOccupancyMaxActiveClusters(&fit, kernel, cfg);
+        if (e == cudaSuccess && fit > 0) return cudaSuccess;
+        if (C == 1) return e == cudaSuccess ? cudaErrorInvalidValue : e;
+        cudaGetLastError();
+        C /= 2;
+    }
 }
 
 template <class T>
@@ -306,6 +466,26 @@ int wave_run_t(long long n, double c, double length, double dt, T *f, T *g, int 
     const T k = T(c * c * dt / (dx * dx));
     // the FP32 energy's factors: (1/2) c^2 (D / (2 dx))^2 dx = K1 D^2, (1/2) (G / 2)^2 dx = K2 G^2
     const double k1 = c * c * dx / (8.0 * dx * dx), k2 = dx / 8.0;
+    if (n <= kClusterCells && n_steps > 0) {
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof cfg);
+        cudaLaunchAttribute attr;
+        if (cluster_config<T>(n, &cfg, &attr, st) == cudaSuccess) {
+            const int C = (int)cfg.gridDim.x, per = (int)((n + C - 1) / C);
+            cudaError_t e = cudaLaunchKernelEx(&cfg, wave_cluster_kernel<T>, f, g, (int)n, per, n_steps,
+                                               T(dt), k, k1, k2, part);
+            if (e == cudaSuccess && energy_out) {
+                wave_cluster_energy_kernel<<<(n_steps + 255) / 256, 256, 0, st>>>(part, C, n_steps, energy);
+                e = cudaGetLastError();
+                if (e == cudaSuccess)
+                    e = cudaMemcpyAsync(energy_out, energy, sizeof(double) * (size_t)n_steps,
+                                        cudaMemcpyDeviceToHost, st);
+            }
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            return e == cudaSuccess ? HYDRO_OK : hydro::record_cuda_error(e, "hydro_wave_run");
+        }
+        cudaGetLastError();  // no cluster fits: the per-step launches
+    }
     // FP32: four cells per thread where n and the arrays allow 128-bit accesses
     const bool vec = sizeof(T) == 4 && n % 4 == 0 && n >= 8 &&
                      reinterpret_cast<uintptr_t>(f) % 16 == 0 && reinterpret_cast<uintptr_t>(g) % 16 == 0 &&
