@@ -731,6 +731,12 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
         else if (strips3(prec, grid->dim, var))
             own_march = hydro::default_strip_planes(grid->n[0], grid->n[1], grid->n[2], sms);
     }
+    if (strips3(prec, grid->dim, var) && variant && variant->march) {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+            own_march = hydro::fitted_strip_planes(grid->n[0], grid->n[1], grid->n[2], var.march, sms);
+    }
     const Layout lay = layout_for(grid->dim, grid->n, ncell, prec, var.manifest);
     if (workspace_bytes < lay.total) return HYDRO_EINVAL;
     // grid-dimension limits of the stage launch

@@ -52,6 +52,8 @@ cudaError_t stage_rows_f32(const StageLaunch &L, cudaStream_t st, bool prepare_o
 // through by default.
 cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only);
 int default_strip_planes(long long nx, long long ny, long long nz, int sm_count);
+// and for a named march of m planes (at most m)
+int fitted_strip_planes(long long nx, long long ny, long long nz, int m, int sm_count);
 int default_strip_rows(long long nx, long long ny, int sm_count);
 
 // Compiled tile shapes (both_pf: both staging depths compiled).

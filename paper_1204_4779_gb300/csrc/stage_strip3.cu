@@ -35,6 +35,23 @@ bool strip3_half_rows(long long nx, long long ny) {
     return strip3_tiles_x<16>(nx) * strip3_tiles_y<16>(ny) < strip3_tiles_x<32>(nx) * strip3_tiles_y<32>(ny);
 }
 
+double strip3_tiles(long long nx, long long ny) {
+    return strip3_half_rows(nx, ny) ? (double)(strip3_tiles_x<16>(nx) * strip3_tiles_y<16>(ny))
+                                    : (double)(strip3_tiles_x<32>(nx) * strip3_tiles_y<32>(ny));
+}
+
+// Modelled time, in planes, of a launch whose CTAs march through m planes (the comment at
+// default_strip_planes).
+double strip3_cost(long long nx, long long ny, long long nz, int m, int sm_count) {
+    const double slots = 2.0 * (sm_count > 0 ? sm_count : 1);
+    const double chunks = (double)((nz + m - 1) / m);
+    double waves = strip3_tiles(nx, ny) * chunks / slots;
+    if (waves >= 6.0)  // by work: the last chunk may be short
+        waves = strip3_tiles(nx, ny) * ((double)nz + 1.5 * chunks) / ((m + 1.5) * slots);
+    const double whole = floor(waves), rest = waves - whole;
+    return (m + 1.5) * (whole + (rest > 0.5 || whole == 0.0 ? 1.0 : (rest > 0.0 ? 0.62 : 0.0)));
+}
+
 template <int SEG> cudaError_t launch_strip3(const StageLaunch &L, StageArgs<float> &A, cudaStream_t st) {
     A.tiles_x = (int)strip3_tiles_x<SEG>(A.n[0]);
     A.tiles_y = (int)strip3_tiles_y<SEG>(A.n[1]);
@@ -68,9 +85,8 @@ cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare
 }
 
 // Planes a CTA marches through when the variant names no march: the least (m + 1.5) x waves, a
-// chunk's prologue counted as 1.5 planes, the waves of the resident CTAs (two per SM) counted by
-// work (the last chunk may be short) with the last one whole, or 0.62 where no SM gets a second
-// CTA of it.  Measured on GB300, blast, us per step at m = 4 / 8 / 12 / 16 / 24 / 32 / 64 / 96,
+// chunk's prologue counted as 1.5 planes, the last wave of the resident CTAs (two per SM) whole,
+// or 0.62 where no SM gets a second CTA of it.  Measured on GB300, blast, us per step at m = 4 / 8 / 12 / 16 / 24 / 32 / 64 / 96,
 // chosen marked:
 //   64^3   30.0* 31.3  40.7  49.9  68.5  86.8  161
 //   128^3  119   116   112   114   110*  142   164   241
@@ -79,18 +95,31 @@ cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare
 //   512^3  5651  5025  4822  4719  4610  4582  4560* 4472
 int default_strip_planes(long long nx, long long ny, long long nz, int sm_count) {
     static const int kPlanes[] = {2, 4, 6, 8, 12, 16, 20, 24, 32, 40, 48, 64, 80, 96, 128};
-    const double tiles = strip3_half_rows(nx, ny)
-                             ? (double)(strip3_tiles_x<16>(nx) * strip3_tiles_y<16>(ny))
-                             : (double)(strip3_tiles_x<32>(nx) * strip3_tiles_y<32>(ny));
-    const double slots = 2.0 * (sm_count > 0 ? sm_count : 1);
     int best = 0;
     double best_cost = 0.0;
-    for (int m : kPlanes) {
-        const double waves =
-            tiles * ((double)nz + 1.5 * (double)((nz + m - 1) / m)) / ((m + 1.5) * slots);
-        const double whole = floor(waves), rest = waves - whole;
-        const double cost = (m + 1.5) * (whole + (rest > 0.5 || whole == 0.0 ? 1.0 : (rest > 0.0 ? 0.62 : 0.0)));
+    for (int named : kPlanes) {
+        const int m = fitted_strip_planes(nx, ny, nz, named, sm_count);
+        const double cost = strip3_cost(nx, ny, nz, m, sm_count);
         if (best == 0 || cost < best_cost) best = m, best_cost = cost;
+    }
+    return best;
+}
+
+// Planes of a CTA for a march of m: over many waves of CTAs m itself (a short last chunk shortens
+// the tail).  Where the chunks make few waves, the waves' rounding and the longest chunk set the
+// time, so the march is an upper bound: of the numbers of chunks that take between m / 2 and m
+// planes each, evenly, the one of least cost (160^3 at 64: three chunks of 54, 54 and 52 planes
+// instead of 64, 64 and 32; at 32: seven of 23 instead of five, which made 1.13 waves).
+int fitted_strip_planes(long long nx, long long ny, long long nz, int m, int sm_count) {
+    const double slots = 2.0 * (sm_count > 0 ? sm_count : 1);
+    const long long least = (nz + m - 1) / m;
+    if (strip3_tiles(nx, ny) * (double)least >= 6.0 * slots) return m;
+    int best = 0;
+    double best_cost = 0.0;
+    for (long long chunks = least; chunks <= 2 * least; ++chunks) {
+        const int k = (int)((nz + chunks - 1) / chunks);
+        const double cost = strip3_cost(nx, ny, nz, k, sm_count);
+        if (best == 0 || cost < best_cost) best = k, best_cost = cost;
     }
     return best;
 }
