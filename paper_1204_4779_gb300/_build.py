@@ -34,6 +34,8 @@ UNITS = {
     "stage_rows.cu": FP32,
     "stage_strip3.cu": FP32,
     "stage_f64.cu": ["--fmad=false"],
+    "line_f32.cu": FP32,
+    "line_f64.cu": ["--fmad=false"],
     "aux_kernels.cu": ["--fmad=false"],
     "hydro_abi.cu": [],
     "static_step.cu": [],
@@ -49,7 +51,7 @@ UNITS = {
 }
 HEADERS = ["hydro_device.cuh", "exact64.cuh", "stage_kernel.cuh", "stage_launch.cuh", "hydro_internal.h",
            "batch_kernel.cuh", "tma.cuh", "pair_device.cuh", "row_kernel.cuh",
-           "strip3_kernel.cuh"]
+           "strip3_kernel.cuh", "line_kernel.cuh"]
 
 
 def nvcc() -> str:

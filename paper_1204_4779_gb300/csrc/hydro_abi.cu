@@ -37,6 +37,7 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr int kMaxChunk = 64;  // largest number of steps captured in one graph
 constexpr int kGraphSlots = 16;
+constexpr int kLineChunk = 2048;  // steps of one launch of a small 1D grid (some 20 ms)
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -326,6 +327,7 @@ struct hydro_ctx {
     void *ex_buf[2][2] = {};
     int ana_kind = 0;        // their solution (hydro_set_analytic); 0 = not set yet
     double ana_theta = 0.0, ana_amp = 0.0;
+    int line_ctas = 0;       // small 1D grids: CTAs of the cluster that runs their steps (0: none)
     double lo[3] = {0, 0, 0};
     void *frame[5] = {};
     hydro_variant_t var = {};
@@ -589,12 +591,30 @@ int run_steps(hydro_ctx *c, const hydro_state_t *s, int n, bool stop_early = fal
     if (c->profiling) return run_steps_profiled(c, s, n);
     int left = n, k = 0;
     while (left > 0) {
-        int chunk = kMaxChunk;
-        while (chunk > left) chunk >>= 1;
-        cudaGraphExec_t g = nullptr;
-        int rc = get_graph(c, s, chunk, &g);
-        if (rc) return rc;
-        CK(cudaGraphLaunch(g, c->stream));
+        int chunk;
+        if (c->line_ctas) {  // a small 1D grid: the chunk's steps in one launch
+            chunk = left < kLineChunk ? left : kLineChunk;
+            hydro::LineLaunch L;
+            for (int a = 0; a < 3; ++a) L.u[a] = s->plane[a];
+            L.n = c->n[0];
+            L.ctas = c->line_ctas;
+            L.periodic = c->periodic[0];
+            L.order = c->order;
+            L.riemann = c->riemann;
+            L.n_steps = chunk;
+            L.dr = c->dr[0];
+            L.gamma = c->gamma;
+            L.ctrl = c->ctrl;
+            CK(c->prec == HYDRO_F32 ? hydro::launch_line_f32(L, c->stream)
+                                    : hydro::launch_line_f64(L, c->stream));
+        } else {
+            chunk = kMaxChunk;
+            while (chunk > left) chunk >>= 1;
+            cudaGraphExec_t g = nullptr;
+            int rc = get_graph(c, s, chunk, &g);
+            if (rc) return rc;
+            CK(cudaGraphLaunch(g, c->stream));
+        }
         left -= chunk;
         if (stop_early && left > 0) {
             const int slot = k & 1;
@@ -815,6 +835,9 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
         delete c;
         return cuda_fail(e, "stage kernel attributes");
     }
+    if (c->dim == 1 && !ana_axes && !ex_axes && c->n[0] >= hydro::kLineLeast &&
+        c->n[0] <= hydro::kLineCells)
+        c->line_ctas = prec == HYDRO_F32 ? hydro::line_ctas_f32(c->n[0]) : hydro::line_ctas_f64(c->n[0]);
     *out = c;
     return HYDRO_OK;
 }

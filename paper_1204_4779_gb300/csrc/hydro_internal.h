@@ -56,6 +56,21 @@ int default_strip_planes(long long nx, long long ny, long long nz, int sm_count)
 int fitted_strip_planes(long long nx, long long ny, long long nz, int m, int sm_count);
 int default_strip_rows(long long nx, long long ny, int sm_count);
 
+// Whole runs of small 1D grids (line_kernel.cuh): up to n_steps steps from the control block's dt
+// on, in one launch.  line_ctas_*: CTAs of the cluster for n cells, 0 if the grid does not fit one.
+constexpr int kLineCells = 2048;  // most cells (least: kLineLeast)
+constexpr int kLineLeast = 32;
+struct LineLaunch {
+    void *u[3];
+    int n, ctas, periodic, order, riemann, n_steps;
+    double dr, gamma;
+    void *ctrl;
+};
+int line_ctas_f32(int n);
+int line_ctas_f64(int n);
+cudaError_t launch_line_f32(const LineLaunch &L, cudaStream_t st);
+cudaError_t launch_line_f64(const LineLaunch &L, cudaStream_t st);
+
 // Compiled tile shapes (both_pf: both staging depths compiled).
 struct TileShape {
     int prec, dim, bx, by, both_pf;
