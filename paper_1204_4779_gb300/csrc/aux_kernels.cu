@@ -141,14 +141,31 @@ __global__ void __launch_bounds__(kAuxThreads)
         for (int k = 0; k < NV; ++k) acc[k] = {0.0f, 0.0f};
         // four cells a thread and access (chunks then start on multiples of four cells)
         const long long q0 = b0 / 4, q1 = A.wide ? b1 / 4 : q0;
-        for (long long q = q0 + threadIdx.x; q < q1; q += kAuxThreads) {
+        // (two groups of four cells in flight; four values are summed exactly in a tree of TwoSums
+        // before they join the running sum: 31 operations instead of 44)
+        auto add4 = [&](int k, const T (&u)[Wide<T>::n]) {
+            const DF p = two_sum((float)u[0], (float)u[1]), r = two_sum((float)u[2], (float)u[3]);
+            const DF h = two_sum(p.hi, r.hi);
+            acc_add(acc[k], {h.hi, h.lo + (p.lo + r.lo)});
+        };
+        long long q = q0 + threadIdx.x;
+        for (; q + kAuxThreads < q1; q += 2 * kAuxThreads) {
+            T u[NV][Wide<T>::n], w[NV][Wide<T>::n];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) load_wide(A.u[k] + 4 * q, u[k]);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) load_wide(A.u[k] + 4 * (q + kAuxThreads), w[k]);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) add4(k, u[k]);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) add4(k, w[k]);
+        }
+        for (; q < q1; q += kAuxThreads) {
             T u[NV][Wide<T>::n];
 #pragma unroll
             for (int k = 0; k < NV; ++k) load_wide(A.u[k] + 4 * q, u[k]);
 #pragma unroll
-            for (int k = 0; k < NV; ++k)
-#pragma unroll
-                for (int c = 0; c < Wide<T>::n; ++c) acc_add(acc[k], {(float)u[k][c], 0.0f});
+            for (int k = 0; k < NV; ++k) add4(k, u[k]);
         }
         for (long long i = (A.wide ? 4 * q1 : b0) + threadIdx.x; i < b1; i += kAuxThreads) {
 #pragma unroll
