@@ -5,7 +5,27 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace hydro {
+
+// Runs `set` (kernel attributes: a property of the process and device) once per device; threads
+// may race to it harmlessly, and a failure is tried again by the next call.
+class PerDevice {
+    std::atomic<unsigned long long> done_{0};
+
+public:
+    template <class F> cudaError_t once(F set) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const unsigned long long bit = 1ull << (dev & 63);
+        if (dev < 64 && (done_.load(std::memory_order_acquire) & bit)) return cudaSuccess;
+        e = set();
+        if (e == cudaSuccess && dev < 64) done_.fetch_or(bit, std::memory_order_release);
+        return e;
+    }
+};
 
 // Record the text of a failed CUDA call for hydro_last_cuda_error(); returns HYDRO_ECUDA.
 int record_cuda_error(cudaError_t e, const char *what);
@@ -19,7 +39,8 @@ struct StageLaunch {
     int n[3];
     int periodic[3];
     int march;
-    int rows;           // FP32 row tiles of dim 2: rows a warp marches through (0: march)
+    int rows;           // strip kernels of dim 2: rows a warp marches through (FP32, 0: march;
+                        // FP64, 0: the tile kernels)
     int tile_x, tile_y;
     int prefetch;       // dim 3: 1 = next plane's loads one plane ahead, 0 = at staging,
                         // 2 = planes staged by TMA (FP32 tiles compiled with it)
@@ -48,6 +69,10 @@ cudaError_t stage_f64(int dim, const StageLaunch &L, cudaStream_t st, bool prepa
 // The FP32 row tiles of dim 2 (stage_rows.cu), and the rows a warp of theirs marches through by
 // default on an nx x ny grid.
 cudaError_t stage_rows_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only);
+// The FP64 strip kernel of dim 2 (stage_row64.cu): the 32 x 8 tile with periodic or outflow
+// boundaries; L.rows rows a warp.
+cudaError_t stage_row64(const StageLaunch &L, cudaStream_t st);
+int default_row64_rows(long long nx, long long ny, int sm_count);
 // The FP32 strip kernels of dim 3 (stage_strip3.cu), and the planes a CTA of theirs marches
 // through by default.
 cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only);

@@ -15,6 +15,8 @@
 // kLineCells the grid kernels, which use every SM, are as fast.
 #pragma once
 
+#include <atomic>
+
 #include "stage_kernel.cuh"
 
 namespace hydro {
@@ -231,33 +233,41 @@ __global__ void __launch_bounds__(kLineThreads) line_kernel(const LineArgs<T> A)
     line_cluster_sync();  // no CTA leaves while another may write to its shared memory
 }
 
-// Cluster of the grid: at most one CTA per 32 cells, a power of two, one cell per thread, as many
-// CTAs as the device runs in one cluster; 0 if there is none.
-template <class T> int line_ctas(int n) {
-    int C = 1;
-    while (C < kLineMaxCtas && n >= 64 * C) C *= 2;
+// The largest cluster of full CTAs the device runs (a property of the kernel and device, asked
+// once per device); 0 if none.
+template <class T> int line_max_ctas() {
+    static std::atomic<int> known[64];  // 1 + the answer
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev < 64 && known[dev].load() > 0) return known[dev].load() - 1;
     const auto k = line_kernel<T>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    for (; C >= 1; C /= 2) {
-        const int per = (n + C - 1) / C;
-        if (per > kLinePer) return 0;
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = (unsigned)C;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)C);
-        cfg.blockDim = dim3((unsigned)(per / 32 * 32 + 32));
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        int fit = 0;
-        if (cudaOccupancyMaxActiveClusters(&fit, k, &cfg) == cudaSuccess && fit > 0) return C;
-        cudaGetLastError();
-    }
-    return 0;
+    int C = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+        for (C = kLineMaxCtas; C >= 1; C /= 2) {
+            cudaLaunchAttribute at;
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = (unsigned)C;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)C);
+            cfg.blockDim = dim3(kLineThreads);
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, k, &cfg) == cudaSuccess && fit > 0) break;
+        }
+    cudaGetLastError();
+    if (dev < 64) known[dev].store(C + 1);
+    return C;
+}
+
+// Cluster of the grid: at most one CTA per 32 cells, a power of two, one cell per thread; 0 if
+// the grid does not fit one.
+template <class T> int line_ctas(int n) {
+    const int most = line_max_ctas<T>();
+    int C = 1;
+    while (2 * C <= most && n >= 64 * C) C *= 2;
+    return most >= 1 && (n + C - 1) / C <= kLinePer ? C : 0;
 }
 
 template <class T> cudaError_t launch_line(const LineLaunch &L, cudaStream_t st) {

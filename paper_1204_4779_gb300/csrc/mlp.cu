@@ -8,7 +8,8 @@
 //
 // Flat parameter layout: W1 (H x d, row-major), b1 (H), W2 (H x H), b2 (H), W3 (1 x H), b3 (1).
 // Workspace for n samples (floats): h1 (n H), h2 (n H), y (n), dy (n), dz2 (n H), dz1 (n H),
-// grad (P), loss (1), the Adam step counter (one int), the weight-gradient chunk partials
+// grad (P), loss (1), the Adam step counter (one int), small networks: what rounding left out of
+// the parameters (P), the weight-gradient chunk partials
 // (ceil(n / kChunk) x H x (max(d, H) + 1)) or, for small networks, the CTAs' gradients and losses.
 //
 // Networks of at most 64 inputs and 64 hidden units (the cost model's) train in two launches per
@@ -35,13 +36,14 @@ constexpr int kChunk = 128;  // samples per partial sum of the weight gradients
 constexpr int kEpochsPerGraph = 16;
 
 struct Sizes {
-    long long P, h1, h2, y, dy, dz2, dz1, grad, loss, stepc, part, total;  // float offsets / count
+    long long P, h1, h2, y, dy, dz2, dz1, grad, loss, stepc, rest, part, total;  // float offsets
 };
 
 constexpr int kSmall = 64;       // most inputs and hidden units of the two-launch epoch
 constexpr int kTile = 32;        // samples of a tile
 constexpr int kTileCtas = 152;   // most CTAs of the tile kernel (one per SM of a GB300)
 constexpr int kRow = kTile + 4;  // floats of a shared row of a tile (rows on distinct banks)
+constexpr int kWRow = kSmall + 1;  // and of a weight matrix (its transposing stores conflict-free)
 
 bool small_net(int d, int H) { return d <= kSmall && H <= kSmall; }
 long long tile_ctas(long long n) {
@@ -62,6 +64,7 @@ Sizes sizes(int d, int H, long long n) {
     S.grad = o; o += S.P;
     S.loss = o; o += 1;
     S.stepc = o; o += 1;
+    S.rest = o; o += small_net(d, H) ? S.P : 0;
     S.part = o;
     const long long chunks = (n + kChunk - 1) / kChunk * (long long)H * ((d > H ? d : H) + 1);
     const long long tiles = small_net(d, H) ? tile_ctas(n) * (S.P + 1) : 0;
@@ -201,7 +204,7 @@ __global__ void __launch_bounds__(kThreads) adam_kernel(float *p, float *m, floa
 // with the input index first for the forward pass, W2 with the output index first for the
 // backward one; a tile's inputs, hidden states and deltas, the sample index last.
 struct TileSmem {
-    float w1[kSmall * kSmall], w2[kSmall * kSmall], w2t[kSmall * kSmall];
+    float w1[kSmall * kWRow], w2[kSmall * kWRow], w2t[kSmall * kWRow];
     float b1[kSmall], b2[kSmall], w3[kSmall];
     float x[kSmall * kRow], h1[kSmall * kRow], h2[kSmall * kRow], z1[kSmall * kRow], z2[kSmall * kRow];
     float dy[kTile], loss[kTile];
@@ -211,7 +214,7 @@ struct TileSmem {
 __device__ __forceinline__ void tile_dense(const float *w, const float *in, int n, int j, int g,
                                            float (&acc)[8]) {
     for (int i = 0; i < n; ++i) {
-        const float c = w[i * kSmall + j];
+        const float c = w[i * kWRow + j];
         const float4 a = *reinterpret_cast<const float4 *>(in + i * kRow + 8 * g);
         const float4 b = *reinterpret_cast<const float4 *>(in + i * kRow + 8 * g + 4);
         acc[0] = fmaf(a.x, c, acc[0]);
@@ -265,14 +268,14 @@ __global__ void __launch_bounds__(kThreads) mlp_tile_kernel(const float *p, int 
     const int P = H * d + H + H * H + H + H + 1;
     const float *W1 = p, *b1 = W1 + H * d, *W2 = b1 + H, *b2 = W2 + H * H, *W3 = b2 + H, *b3 = W3 + H;
     if (stepc && blockIdx.x == 0 && tid == 0) *stepc += 1;
-    for (int q = tid; q < kSmall * kSmall; q += kThreads) M.w1[q] = M.w2[q] = M.w2t[q] = 0.0f;
+    for (int q = tid; q < kSmall * kWRow; q += kThreads) M.w1[q] = M.w2[q] = M.w2t[q] = 0.0f;
     for (int q = tid; q < kSmall * kRow; q += kThreads) M.x[q] = 0.0f;
     __syncthreads();
-    for (int q = tid; q < H * d; q += kThreads) M.w1[(q % d) * kSmall + q / d] = W1[q];
+    for (int q = tid; q < H * d; q += kThreads) M.w1[(q % d) * kWRow + q / d] = W1[q];
     for (int q = tid; q < H * H; q += kThreads) {
         const float w = W2[q];
-        M.w2[(q % H) * kSmall + q / H] = w;
-        M.w2t[(q / H) * kSmall + q % H] = w;
+        M.w2[(q % H) * kWRow + q / H] = w;
+        M.w2t[(q / H) * kWRow + q % H] = w;
     }
     if (tid < kSmall) {
         M.b1[tid] = tid < H ? b1[tid] : 0.0f;
@@ -374,12 +377,14 @@ __global__ void __launch_bounds__(kThreads) mlp_tile_kernel(const float *p, int 
 constexpr int kUpdateParams = 32;  // parameters of an update CTA, eight threads each
 
 // grad = the sum of the tile CTAs' gradients, eight runs of CTAs in parallel, the runs in order;
-// then, training (stepc non-null), the Adam update of adam_kernel_dev.  The thread of index P
-// sums the losses.
+// then, training (stepc non-null), the Adam update of adam_kernel_dev, with what rounding a
+// parameter to FP32 leaves out carried to its next update (rest; TwoSum): an update of about lr is
+// 1e-3 of a parameter, and without that 200 updates' roundings are most of the result's error.
+// The thread of index P sums the losses.
 __global__ void __launch_bounds__(kThreads)
     mlp_update_kernel(const float *part, int ctas, int P, long long n, float *grad, float *loss_out,
-                      float *p, float *m, float *v, float lr, float b1, float b2, float eps,
-                      const int *stepc, int step0, float *hist) {
+                      float *p, float *m, float *v, float *rest, float lr, float b1, float b2,
+                      float eps, const int *stepc, int step0, float *hist) {
     __shared__ float run[8][kUpdateParams];
     const int q = threadIdx.x & (kUpdateParams - 1), r = threadIdx.x / kUpdateParams;
     const int i = blockIdx.x * kUpdateParams + q;
@@ -408,7 +413,10 @@ __global__ void __launch_bounds__(kThreads)
     const float vi = b2 * v[i] + (1.0f - b2) * acc * acc;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / k1) / (sqrtf(vi / k2) + eps);
+    const float q0 = p[i], y = __fadd_rn(rest[i], -(lr * (mi / k1) / (sqrtf(vi / k2) + eps)));
+    const float q1 = __fadd_rn(q0, y), back = __fadd_rn(q1, -q0);
+    rest[i] = __fadd_rn(__fadd_rn(q0, -__fadd_rn(q1, -back)), __fadd_rn(y, -back));
+    p[i] = q1;
 }
 
 // One small-network epoch (or, with m null, the gradient alone).
@@ -419,13 +427,16 @@ cudaError_t small_epoch(float *p, float *m, float *v, int d, int H, const float 
     float *part = ws + S.part;
     mlp_tile_kernel<<<ctas, kThreads, sizeof(TileSmem), st>>>(p, d, H, X, t, n, part, stepc);
     mlp_update_kernel<<<(P + 1 + kUpdateParams - 1) / kUpdateParams, kThreads, 0, st>>>(
-        part, ctas, P, n, ws + S.grad, ws + S.loss, p, m, v, lr, 0.9f, 0.999f, 1e-8f, stepc, step0,
-        hist);
+        part, ctas, P, n, ws + S.grad, ws + S.loss, p, m, v, ws + S.rest, lr, 0.9f, 0.999f, 1e-8f,
+        stepc, step0, hist);
     return cudaGetLastError();
 }
 cudaError_t small_prepare() {
-    return cudaFuncSetAttribute(mlp_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sizeof(TileSmem));
+    static hydro::PerDevice attribute;
+    return attribute.once([] {
+        return cudaFuncSetAttribute(mlp_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sizeof(TileSmem));
+    });
 }
 
 unsigned blocks(long long work) { return (unsigned)((work + kThreads - 1) / kThreads); }
@@ -558,6 +569,7 @@ int hydro_mlp_train(float *params, float *m, float *v, int32_t d, int32_t hidden
     cudaError_t e = cudaGetLastError();
     if (small_net(d, hidden)) {  // two launches an epoch: the GPU, not the launches, sets the pace
         if (e == cudaSuccess) e = small_prepare();
+        if (e == cudaSuccess) e = cudaMemsetAsync(ws + S.rest, 0, sizeof(float) * (size_t)S.P, st);
         for (int k = 0; k < epochs && e == cudaSuccess; ++k)
             e = small_epoch(params, m, v, d, hidden, X, t, n, ws, S, lr, stepc, step0, loss_out, st);
         return e == cudaSuccess ? HYDRO_OK : hydro::record_cuda_error(e, "hydro_mlp_train");

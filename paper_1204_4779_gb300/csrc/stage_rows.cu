@@ -61,9 +61,12 @@ int row_march(long long strips, long long ny, int warp_slots) {
 cudaError_t stage_rows_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only) {
     if (L.tile_x % 64 != 0 || L.tile_x > 64 * (kRowThreads / 32)) return cudaErrorInvalidValue;
     if (prepare_only) {
-        cudaError_t e = RowKernels<1, false>::prepare();
-        if (e == cudaSuccess) e = RowKernels<2, false>::prepare();
-        return e == cudaSuccess ? RowKernels<2, true>::prepare() : e;
+        static PerDevice attributes;
+        return attributes.once([] {
+            cudaError_t e = RowKernels<1, false>::prepare();
+            if (e == cudaSuccess) e = RowKernels<2, false>::prepare();
+            return e == cudaSuccess ? RowKernels<2, true>::prepare() : e;
+        });
     }
     StageArgs<float> A = make_stage_args<float>(L);
     const long long strips = (A.n[0] + kStripCells - 1) / kStripCells;

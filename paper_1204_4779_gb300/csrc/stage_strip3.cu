@@ -72,12 +72,15 @@ template <int SEG> cudaError_t launch_strip3(const StageLaunch &L, StageArgs<flo
 
 cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare_only) {
     if (prepare_only) {
-        cudaError_t e = Strip3Kernels<32, 1, false>::prepare();
-        if (e == cudaSuccess) e = Strip3Kernels<32, 2, false>::prepare();
-        if (e == cudaSuccess) e = Strip3Kernels<32, 2, true>::prepare();
-        if (e == cudaSuccess) e = Strip3Kernels<16, 1, false>::prepare();
-        if (e == cudaSuccess) e = Strip3Kernels<16, 2, false>::prepare();
-        return e == cudaSuccess ? Strip3Kernels<16, 2, true>::prepare() : e;
+        static PerDevice attributes;
+        return attributes.once([] {
+            cudaError_t e = Strip3Kernels<32, 1, false>::prepare();
+            if (e == cudaSuccess) e = Strip3Kernels<32, 2, false>::prepare();
+            if (e == cudaSuccess) e = Strip3Kernels<32, 2, true>::prepare();
+            if (e == cudaSuccess) e = Strip3Kernels<16, 1, false>::prepare();
+            if (e == cudaSuccess) e = Strip3Kernels<16, 2, false>::prepare();
+            return e == cudaSuccess ? Strip3Kernels<16, 2, true>::prepare() : e;
+        });
     }
     StageArgs<float> A = make_stage_args<float>(L);
     return strip3_half_rows(A.n[0], A.n[1]) ? launch_strip3<16>(L, A, st)

@@ -41,6 +41,8 @@
 // FP64 evaluation of the FP32 state's energy to about 2^-48 times the cells a thread visits.
 #include <string.h>
 
+#include <atomic>
+
 #include "../../include/hydro.h"
 #include "hydro_device.cuh"
 #include "hydro_internal.h"
@@ -423,20 +425,12 @@ WaveLayout wave_layout(long long n, int prec, int n_steps) {
     return L;
 }
 
-// CTAs of the cluster for n cells: at most one per 64 cells, a power of two, and as many as the
-// device runs at once.
-template <class T> cudaError_t cluster_config(long long n, cudaLaunchConfig_t *cfg,
-                                              cudaLaunchAttribute *attr, cudaStream_t st) {
-    int C = 1;
-    while (C < kClusterMax && n >= 64LL * 2 * C) C *= 2;
+// The launch of the cluster kernel for n cells: at most one CTA per 64 cells, a power of two, and
+// no more than the device runs as one cluster of full CTAs (asked once per device).
+template <class T> bool cluster_config(long long n, cudaLaunchConfig_t *cfg,
+                                       cudaLaunchAttribute *attr, cudaStream_t st) {
     const auto kernel = wave_cluster_kernel<T>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    for (;;) {
-        const long long per = (n + C - 1) / C;
-        long long threads = (per + 31) / 32 * 32;
-        if (threads > kClusterThreads) threads = kClusterThreads;
-        if (per > threads * kClusterPer) return cudaErrorInvalidValue;
+    auto set = [&](int C, int threads) {
         attr->id = cudaLaunchAttributeClusterDimension;
         attr->val.clusterDim.x = (unsigned)C;
         attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
@@ -446,13 +440,30 @@ template <class T> cudaError_t cluster_config(long long n, cudaLaunchConfig_t *c
         cfg->stream = st;
         cfg->attrs = attr;
         cfg->numAttrs = 1;
-        int fit = 0;
-        e = cudaOccupancyMaxActiveClusters(&fit, kernel, cfg);
-        if (e == cudaSuccess && fit > 0) return cudaSuccess;
-        if (C == 1) return e == cudaSuccess ? cudaErrorInvalidValue : e;
+    };
+    static std::atomic<int> known[64];  // 1 + the largest cluster
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return false;
+    int most = known[dev].load() - 1;
+    if (most < 0) {
+        most = 0;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+            for (most = kClusterMax; most >= 1; most /= 2) {
+                int fit = 0;
+                set(most, kClusterThreads);
+                if (cudaOccupancyMaxActiveClusters(&fit, kernel, cfg) == cudaSuccess && fit > 0) break;
+            }
         cudaGetLastError();
-        C /= 2;
+        known[dev].store(most + 1);
     }
+    int C = 1;
+    while (2 * C <= most && n >= 64LL * 2 * C) C *= 2;
+    const long long per = (n + C - 1) / C;
+    long long threads = (per + 31) / 32 * 32;
+    if (threads > kClusterThreads) threads = kClusterThreads;
+    if (most < 1 || per > threads * kClusterPer) return false;
+    set(C, (int)threads);
+    return true;
 }
 
 template <class T>
@@ -470,7 +481,7 @@ int wave_run_t(long long n, double c, double length, double dt, T *f, T *g, int 
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof cfg);
         cudaLaunchAttribute attr;
-        if (cluster_config<T>(n, &cfg, &attr, st) == cudaSuccess) {
+        if (cluster_config<T>(n, &cfg, &attr, st)) {
             const int C = (int)cfg.gridDim.x, per = (int)((n + C - 1) / C);
             cudaError_t e = cudaLaunchKernelEx(&cfg, wave_cluster_kernel<T>, f, g, (int)n, per, n_steps,
                                                T(dt), k, k1, k2, part);
@@ -484,7 +495,6 @@ int wave_run_t(long long n, double c, double length, double dt, T *f, T *g, int 
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             return e == cudaSuccess ? HYDRO_OK : hydro::record_cuda_error(e, "hydro_wave_run");
         }
-        cudaGetLastError();  // no cluster fits: the per-step launches
     }
     // FP32: four cells per thread where n and the arrays allow 128-bit accesses
     const bool vec = sizeof(T) == 4 && n % 4 == 0 && n >= 8 &&
