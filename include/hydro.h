@@ -100,6 +100,11 @@ typedef struct {
  *                   (tile, chunk) work items fill the GPU's resident CTAs three times (row
  *                   tiles: twice), the one with the least 0.5 x chunks + 0.3 x planes of the
  *                   last chunk, else 8 (row tiles: 16); FP64: 64 in dim 3, 16 for row tiles).
+ *                   Where no march is named, the FP32 strip kernels (below) and the FP64 3D
+ *                   tiles choose the planes of a chunk themselves from the grid and the GPU, and
+ *                   hydro_get_variant reports the default above.  On the 3D strip kernels a
+ *                   named march is an upper bound where its chunks make fewer than three waves
+ *                   of CTAs: they take between half of it and all of it, evenly.
  *   split:          fusion split.  0 = library default (fused for marching tiles, separate
  *                   for one-plane tiles); 1 = a separate CFL pass after RK stage 2 (one more
  *                   launch and one more read of the state per step); 2 = the CFL signal and
@@ -129,6 +134,11 @@ typedef struct {
  *                   16 x 8, 32 x 8, 16 x 16; FP64 32 x 8), with look-ahead staging and the
  *                   precision's default budget; 2 and 3 need more workspace
  *                   (hydro_workspace_bytes_variant).
+ * Strip kernels: the FP32 row tiles of dim 2 and, in dim 3, the FP32 tile 16 x 8 with look-ahead
+ * staging and nothing manifest run kernels whose warps own strips of 64 columns, two cells per
+ * lane, and march with everything in registers.  Of a row tile's width they take one warp per 64
+ * columns; staging and occupancy do not apply to them.  Grids of dim 1 of 32 to 2048 cells with
+ * periodic or outflow ends run whole chunks of steps in one launch, whatever the variant.
  * Library defaults (measured on GB300): dim 3 FP32 tile 16 x 8 (march from the grid size: 96
  * at 512^3), FP64 32 x 8, march 64; dim 2 FP32 row tile 256 x 1 (march from the grid size: 16
  * at 2048^2, 64 at 4096^2); dim 2 FP64 tile 32 x 8; dim 1 tile 128.  A variant that names a tile other than the default gets that
@@ -245,7 +255,7 @@ int hydro_set_scheme(hydro_ctx_t *ctx, int32_t order, int32_t riemann);
  * dt is computed on the device from the state at the start of each step (the first from
  * `state` by a CFL pass, later ones in the epilogue of the previous step) and never leaves
  * the device inside the call.  The steps run as CUDA graphs of captured launches (chunks of up
- * to 64 steps); once no further step is to be taken (t_end reached or a failed step) the steps
+ * to 64 steps; grids of dim 1 of 32 to 2048 cells: up to 2048 steps in one launch); once no further step is to be taken (t_end reached or a failed step) the steps
  * left return at once on the device, and a synchronous call stops launching chunks after
  * that (it reads dt back after each chunk, one chunk late, so n_steps may be a generous
  * bound when t_end is what ends the run).

@@ -34,6 +34,7 @@ UNITS = {
     "stage_rows.cu": FP32,
     "stage_strip3.cu": FP32,
     "stage_f64.cu": ["--fmad=false"],
+    "stage_row64.cu": ["--fmad=false"],
     "line_f32.cu": FP32,
     "line_f64.cu": ["--fmad=false"],
     "aux_kernels.cu": ["--fmad=false"],
@@ -51,7 +52,7 @@ UNITS = {
 }
 HEADERS = ["hydro_device.cuh", "exact64.cuh", "stage_kernel.cuh", "stage_launch.cuh", "hydro_internal.h",
            "batch_kernel.cuh", "tma.cuh", "pair_device.cuh", "row_kernel.cuh",
-           "strip3_kernel.cuh", "line_kernel.cuh"]
+           "strip3_kernel.cuh", "line_kernel.cuh", "row64_kernel.cuh"]
 
 
 def nvcc() -> str:

@@ -142,11 +142,11 @@ int tile_compiled_tma(int prec, int dim, int bx, int by) {
     return 0;
 }
 
-// Defaults chosen by measurements on GB300.  dim 3: marching 64 planes; FP32 tile 16 x 8 with
-// the three-CTA register budget (the variant tuner's best: 23.03 against 22.82 G
-// cell-updates/s for 32 x 8 at 512^3), FP64 tile 32 x 8 (its one compiled 3D tile).  dim 2, FP32: row tiles of 256
-// cells marching 16 rows along y, three-CTA budget (2048^2: 28.4 G cell-updates/s against 20.8
-// G for the best one-plane tile).  dim 1 and FP64 dim 2: one-plane tiles.  The dt reduction is
+// Defaults chosen by measurements on GB300.  dim 3: FP32 tile 16 x 8, which runs the strip kernels
+// (512^3: 30 G cell-updates/s against 23.4 G for the shared-memory tiles), FP64 tile 32 x 8 (its
+// one compiled 3D tile), marching 64 planes.  dim 2, FP32: row tiles, which run the strip kernels
+// (2048^2: 42 G cell-updates/s against 30.2 G for the shared-memory rows and 20.8 G for the best
+// one-plane tile).  dim 1 and FP64 dim 2: one-plane tiles.  The dt reduction is
 // fused into stage 2 for marching tiles; for one-plane tiles, where a CTA updates one tile, the
 // separate CFL pass (a fused per-CTA reduction costs more there than one extra read of the
 // state).  The split is settled in resolve_variant, once the tile is known.
@@ -177,16 +177,12 @@ void default_variant(int prec, int dim, hydro_variant_t *v) {
     }
 }
 
-// Default march of a 3D FP32 grid (a variant that names no march).  A CTA advances one tile
-// through `march` planes after a short prologue; the launch's (tile, chunk) work items run in
-// order, chunk by chunk, so the last chunk's items (shorter where the march does not divide
-// the extent) finish the launch.  Among marches 8, 16, 32, ..., 128 whose items fill the GPU's
-// resident CTAs at least three times, the one with the least modelled overhead: 0.5 plane per
-// chunk (the prologue) plus 0.3 times the last chunk's planes (the launch's tail); 8 when none
-// fills them three times.  The weights were fitted to blast runs on GB300 (marches 16-128, n =
-// 256 ... 640); G cell-updates/s, the chosen march marked: 512^3 23.14 (64) 23.29 (80) 23.32
-// (96*); 448^3 22.90 (64) 23.25 (48*); 384^3 22.62 (64) 22.87 (32*); 256^3 20.56 (64) 21.85
-// (16) 22.08 (48*); 128^3 11.56 (64) 15.74 (16) 17.41 (8*).
+// Reported default march of a 3D FP32 grid (a variant that names no march; the shared-memory tiles
+// run it, the strip kernels take hydro::default_strip_planes): among marches 8, 16, 32, ..., 128
+// whose items fill the GPU's resident CTAs at least three times, the one with the least modelled
+// overhead: 0.5 plane per chunk (the prologue) plus 0.3 times the last chunk's planes (the
+// launch's tail); 8 when none fills them three times.  The weights were fitted to the
+// shared-memory tiles' blast runs on GB300 (marches 16-128, n = 256 ... 640).
 // The march of `tiles` tiles marching through `extent` planes: among `marches` those whose
 // work items fill `slots` resident CTAs `waves` times, the one with the least
 // 0.5 chunks + 0.3 (planes of the last chunk); `fallback` when none does.
@@ -240,12 +236,10 @@ int default_march_f64_3d(const int64_t n[3], const hydro_variant_t &v, int sm_co
     return best;
 }
 
-// Default march of the 2D FP32 row tiles (a variant that names no march), with the same cost
-// and marches 8, 16, 32, 64, 128 whose items fill the resident CTAs twice (launches of more
-// items than resident CTAs run persistently, so a short last wave costs little); 16 when none
-// does.  Measured on GB300 (shear layer, tile 256 x 1, G cell-updates/s, marches 8 / 16 / 32 /
-// 64, chosen marked): 4096^2 32.3 / 34.3 / 34.0 / 35.6*; 2048^2 28.4 / 30.2* / 25.6 / 24.9;
-// 1024^2 (no march fills them twice) 19.5 / 20.4* / 15.5 / -.
+// Reported default march of the 2D FP32 row tiles (a variant that names no march), with the same
+// cost and marches 8, 16, 32, 64, 128 whose items fill the resident CTAs twice; 16 when none does.
+// It is what hydro_get_variant names; a warp of the strip kernels takes
+// hydro::default_strip_rows instead.
 int default_march_rows(const int64_t n[3], const hydro_variant_t &v, int sm_count) {
     static const int kMarch[] = {8, 16, 32, 64, 128};
     const long long strips = (n[0] + v.tile_x - 1) / v.tile_x;
@@ -331,7 +325,9 @@ struct hydro_ctx {
     double lo[3] = {0, 0, 0};
     void *frame[5] = {};
     hydro_variant_t var = {};
-    int strip_rows = 0;      // FP32 row tiles without a named march: rows of a warp
+    int strip_rows = 0;      // rows of a warp of the strip kernels of dim 2: FP32 row tiles without
+                             // a named march, the FP64 32 x 8 tile
+    int split = 0;           // 1: a separate CFL pass after stage 2
     int march = 1;           // planes of a chunk: the variant's, or where it names none the
                              // choice of the 3D strip kernels or of the FP64 tiles
     Layout lay = {};
@@ -383,7 +379,7 @@ hydro::StageLaunch stage_args(const hydro_ctx *c, const hydro_state_t *s, int st
     L.tile_x = c->var.tile_x;
     L.tile_y = c->var.tile_y;
     L.prefetch = c->var.staging == 2 ? 0 : (c->var.staging == 3 ? 2 : 1);
-    L.split = c->var.split;
+    L.split = c->split;
     L.occupancy = c->var.occupancy;
     L.manifest = c->var.manifest == 2 ? 1 : (c->var.manifest == 3 ? 2 : 0);
     for (int k = 0; k < 5; ++k) L.vbuf[k] = c->vbuf[k];
@@ -515,7 +511,7 @@ int get_graph(hydro_ctx *c, const hydro_state_t *s, int chunk, cudaGraphExec_t *
     for (int i = 0; i < chunk && le == cudaSuccess; ++i) {
         le = launch_stage(c, L1, c->cap);
         if (le == cudaSuccess) le = launch_stage(c, L2, c->cap);
-        if (le == cudaSuccess && c->var.split) le = hydro::launch_cfl(C, c->cap, /*advance=*/true);
+        if (le == cudaSuccess && c->split) le = hydro::launch_cfl(C, c->cap, /*advance=*/true);
     }
     cudaGraph_t graph = nullptr;
     cudaError_t ee = cudaStreamEndCapture(c->cap, &graph);
@@ -542,7 +538,7 @@ int get_graph(hydro_ctx *c, const hydro_state_t *s, int chunk, cudaGraphExec_t *
 int run_steps_profiled(hydro_ctx *c, const hydro_state_t *s, int n) {
     const hydro::StageLaunch L1 = stage_args(c, s, 1), L2 = stage_args(c, s, 2);
     const hydro::AuxArgs C = aux_args(c, s);
-    const int per = c->var.split ? 3 : 2;  // launches per step
+    const int per = c->split ? 3 : 2;  // launches per step
     const size_t need = (size_t)per * kMaxChunk + 1;
     while (c->events.size() < need) {
         cudaEvent_t e;
@@ -558,7 +554,7 @@ int run_steps_profiled(hydro_ctx *c, const hydro_state_t *s, int n) {
             CK(cudaEventRecord(c->events[e0 + 1], c->stream));
             CK(launch_stage(c, L2, c->stream));
             CK(cudaEventRecord(c->events[e0 + 2], c->stream));
-            if (c->var.split) {
+            if (c->split) {
                 CK(hydro::launch_cfl(C, c->stream, /*advance=*/true));
                 CK(cudaEventRecord(c->events[e0 + 3], c->stream));
             }
@@ -734,6 +730,13 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
     }
     const bool rows = grid->dim == 2 && var.tile_y == 1;
     int strip_rows = 0, own_march = 0;
+    if (grid->dim == 2 && prec == HYDRO_F64 && var.tile_x == 32 && var.tile_y == 8 &&
+        !(ana_axes | ex_axes)) {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+            strip_rows = hydro::default_row64_rows(grid->n[0], grid->n[1], sms);
+    }
     if (grid->dim == 3 && prec == HYDRO_F64 && !(variant && variant->march)) {
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -790,6 +793,9 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
     c->cfl = cfl;
     c->var = var;
     c->strip_rows = strip_rows;
+    // the FP64 strips keep the new states in registers: the dt reduction joins stage 2 unless the
+    // variant names the separate pass (the reported default belongs to the tile kernels)
+    c->split = strip_rows && prec == HYDRO_F64 && !(variant && variant->split) ? 0 : var.split;
     c->march = own_march ? own_march : var.march;
     if (marching && c->march > c->n[c->dim - 1]) c->march = c->n[c->dim - 1];
     c->lay = lay;

@@ -8,6 +8,8 @@ cudaError_t stage_f64(int dim, const StageLaunch &L, cudaStream_t st, bool prepa
     if (dim == 1) {
         HYDRO_STAGE_CASE(double, 1, 128, 1, false)
     } else if (dim == 2) {
+        if (L.tile_x == 32 && L.tile_y == 8 && L.rows > 0 && !L.ana && !prepare_only)
+            return stage_row64(L, st);
         HYDRO_STAGE_CASE(double, 2, 32, 8, false)
         HYDRO_STAGE_CASE(double, 2, 128, 1, false)
     } else if (dim == 3) {

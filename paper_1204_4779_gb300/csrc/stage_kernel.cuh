@@ -1,4 +1,5 @@
-// Fused RK-stage kernel of the compressible-Euler step (arXiv:1204.4779, section 4.1).
+// Fused RK-stage kernel of the compressible-Euler step (arXiv:1204.4779, section 4.1): FP64, and the
+// FP32 tiles other than the strips (row_kernel.cuh, strip3_kernel.cuh), which are the defaults.
 //
 // One launch computes, for every cell i,
 //     U_out[i] = U_base[i] + sum_a (c dt / dr_a) (F_a[i - e_a/2] - F_a[i + e_a/2]),
@@ -804,7 +805,7 @@ __global__ void __launch_bounds__(BX * BY, (MinBlocks<T, BX * BY, OCC>::value))
 // CTA b takes item b, then claims the next unclaimed item from the control block's counter
 // until none is left, so the last wave of a launch with few items per SM does not leave SMs
 // idle.  The last CTA to stop claiming resets the counters for the next launch on the same
-// control block.  Used where the items make only a few waves of CTAs (the row tiles of 2D
+// control block.  Used where the items make only a few waves of CTAs (the FP64 row tiles of 2D
 // grids): over many waves the hardware's own scheduling loses nothing and the claiming loop
 // costs instructions.
 template <class T, int D, int BX, int BY, int STAGE, int PF, bool FUSED = true, int OCC = 2>
