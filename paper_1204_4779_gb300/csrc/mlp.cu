@@ -8,20 +8,20 @@
 //
 // Flat parameter layout: W1 (H x d, row-major), b1 (H), W2 (H x H), b2 (H), W3 (1 x H), b3 (1).
 // Workspace for n samples (floats): h1 (n H), h2 (n H), y (n), dy (n), dz2 (n H), dz1 (n H),
-// grad (P), loss (1), the Adam step counter (one int), small networks: what rounding left out of
-// the parameters (P), the weight-gradient chunk partials
-// (ceil(n / kChunk) x H x (max(d, H) + 1)) or, for small networks, the CTAs' gradients and losses.
+// grad (P), loss (1), the Adam step counter (one int), the weight-gradient chunk partials
+// (ceil(n / kChunk) x H x (max(d, H) + 1), or x P for small networks).
 //
 // Networks of at most 64 inputs and 64 hidden units (the cost model's) train in two launches per
-// epoch: mlp_tile_kernel takes tiles of 32 samples through forward pass, loss and
-// back-propagation in shared memory and leaves each CTA's weight gradients; mlp_update_kernel sums
-// them in CTA order and applies Adam.  The thirteen launches of the general kernels took 174 us an
-// epoch (4200 records, 35 inputs, width 64), most of it in gathers and launches; the two take
-// about 9.  The general kernels serve wider networks.
+// epoch: mlp_chunk_kernel takes a chunk of samples through forward pass and back-propagation in
+// the shared memory of a thread-block cluster and leaves the chunk's weight gradients;
+// mlp_update_kernel sums them in chunk order and applies Adam.  The thirteen launches of the
+// general kernels took 174 us an epoch (4200 records, 35 inputs, width 64), most of it in gathers
+// and launches; the two take 27, with equal bits.  The general kernels serve wider networks.
 //
 // There training replays captured epochs: the Adam step number lives in the workspace (the loss
 // kernel advances it, the Adam kernel derives its bias corrections from it), so one epoch's
 // launches are the same every epoch and a CUDA graph of kEpochsPerGraph epochs is replayed.
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
@@ -30,26 +30,27 @@
 
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kThreads = 256;
 constexpr int kChunk = 128;  // samples per partial sum of the weight gradients
 
 constexpr int kEpochsPerGraph = 16;
 
 struct Sizes {
-    long long P, h1, h2, y, dy, dz2, dz1, grad, loss, stepc, rest, part, total;  // float offsets
+    long long P, h1, h2, y, dy, dz2, dz1, grad, loss, stepc, part, total;  // float offsets
 };
 
-constexpr int kSmall = 64;       // most inputs and hidden units of the two-launch epoch
-constexpr int kTile = 32;        // samples of a tile
-constexpr int kTileCtas = 152;   // most CTAs of the tile kernel (one per SM of a GB300)
-constexpr int kRow = kTile + 4;  // floats of a shared row of a tile (rows on distinct banks)
-constexpr int kWRow = kSmall + 1;  // and of a weight matrix (its transposing stores conflict-free)
+constexpr int kSmall = 64;                // most inputs and hidden units of the two-launch epoch
+constexpr int kTile = 32;                 // samples of a CTA's tile
+constexpr int kTiles = kChunk / kTile;    // CTAs of a cluster
+constexpr int kUnits = kSmall / kTiles;   // units whose gradients a CTA sums
+constexpr int kChunkThreads = kThreads + 32;
+constexpr int kRow = kTile + 4;           // floats of a shared row of a tile,
+constexpr int kCRow = kChunk + 4;         // of a chunk (rows on distinct banks)
+constexpr int kWRow = kSmall + 1;         // and of a weight matrix (either index conflict-free)
 
 bool small_net(int d, int H) { return d <= kSmall && H <= kSmall; }
-long long tile_ctas(long long n) {
-    const long long t = (n + kTile - 1) / kTile;
-    return t < kTileCtas ? t : kTileCtas;
-}
 
 Sizes sizes(int d, int H, long long n) {
     Sizes S;
@@ -64,11 +65,9 @@ Sizes sizes(int d, int H, long long n) {
     S.grad = o; o += S.P;
     S.loss = o; o += 1;
     S.stepc = o; o += 1;
-    S.rest = o; o += small_net(d, H) ? S.P : 0;
     S.part = o;
-    const long long chunks = (n + kChunk - 1) / kChunk * (long long)H * ((d > H ? d : H) + 1);
-    const long long tiles = small_net(d, H) ? tile_ctas(n) * (S.P + 1) : 0;
-    o += chunks > tiles ? chunks : tiles;
+    const long long per = (long long)H * ((d > H ? d : H) + 1);
+    o += (n + kChunk - 1) / kChunk * (small_net(d, H) && S.P > per ? S.P : per);
     S.total = o;
     return S;
 }
@@ -87,6 +86,17 @@ __global__ void __launch_bounds__(kThreads) dense_forward(const float *in, int d
     out[idx] = TANH ? tanhf(acc) : acc;
 }
 
+// The sum of the CTA's kThreads values by halving, in thread 0
+__device__ __forceinline__ float block_sum(float (&s)[kThreads], float value) {
+    s[threadIdx.x] = value;
+    __syncthreads();
+    for (int w = kThreads / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
+        __syncthreads();
+    }
+    return s[0];
+}
+
 // dy[s] = 2 (y[s] - t[s]) / n; loss = (1/n) sum_s (y[s] - t[s])^2 (one CTA, fixed order).
 // Training (stepc non-null): also record the loss in hist[*stepc - step0] and advance the Adam
 // step counter *stepc, which the Adam kernel of the same epoch reads.
@@ -100,16 +110,11 @@ __global__ void __launch_bounds__(kThreads) mse_kernel(const float *y, const flo
         dy[i] = 2.0f * e / (float)n;
         acc = fmaf(e, e, acc);
     }
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
-        __syncthreads();
-    }
+    const float sum = block_sum(s, acc);
     if (threadIdx.x == 0) {
-        *loss = s[0] / (float)n;
+        *loss = sum / (float)n;
         if (stepc) {
-            if (hist) hist[*stepc - step0] = s[0] / (float)n;
+            if (hist) hist[*stepc - step0] = sum / (float)n;
             *stepc += 1;
         }
     }
@@ -166,21 +171,25 @@ __global__ void __launch_bounds__(kThreads) dense_wgrad_sum(const float *part, i
         gb[j] = acc;
 }
 
-// Adam with the step number t = *stepc read on the device (bias corrections 1 - b^t)
+// Adam's step number t for parameter i of gradient gi (bias corrections 1 - b^t)
+__device__ __forceinline__ void adam_step(float *p, float *m, float *v, long long i, float gi,
+                                          float lr, float b1, float b2, float eps, float t) {
+    const float c1 = 1.0f - powf(b1, t), c2 = 1.0f - powf(b2, t);
+    const float mi = b1 * m[i] + (1.0f - b1) * gi;
+    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+    m[i] = mi;
+    v[i] = vi;
+    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+
+// Adam with the step number read on the device
 __global__ void __launch_bounds__(kThreads) adam_kernel_dev(float *p, float *m, float *v,
                                                             const float *g, long long count,
                                                             float lr, float b1, float b2, float eps,
                                                             const int *stepc) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
-    const float t = (float)*stepc;
-    const float c1 = 1.0f - powf(b1, t), c2 = 1.0f - powf(b2, t);
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    adam_step(p, m, v, i, g[i], lr, b1, b2, eps, (float)*stepc);
 }
 
 __global__ void set_step_kernel(int *stepc, int value) { *stepc = value; }
@@ -200,23 +209,27 @@ __global__ void __launch_bounds__(kThreads) adam_kernel(float *p, float *m, floa
 
 // ---- the two-launch epoch -------------------------------------------------------------------
 
-// Shared memory of the tile kernel (floats): the weights padded to 64 x 64 with zeros, W1 and W2
-// with the input index first for the forward pass, W2 with the output index first for the
-// backward one; a tile's inputs, hidden states and deltas, the sample index last.
-struct TileSmem {
-    float w1[kSmall * kWRow], w2[kSmall * kWRow], w2t[kSmall * kWRow];
+// Shared memory of the chunk kernel (floats).  Weights with the input index first; a tile's own
+// rows (z2, h2) of 32 samples; rows of the chunk's 128 samples, the sample index last: the inputs
+// and first hidden states of all units, and for the CTA's 16 units the deltas and second states.
+struct ChunkSmem {
+    float w1[kSmall * kWRow], w2[kSmall * kWRow];
     float b1[kSmall], b2[kSmall], w3[kSmall];
-    float x[kSmall * kRow], h1[kSmall * kRow], h2[kSmall * kRow], z1[kSmall * kRow], z2[kSmall * kRow];
-    float dy[kTile], loss[kTile];
+    float x[kSmall * kCRow], h1[kSmall * kCRow];
+    float h2[kSmall * kRow], z2[kSmall * kRow];
+    float z1c[kUnits * kCRow], z2c[kUnits * kCRow], h2c[kUnits * kCRow];
+    float dy[kChunk];
 };
 
-// acc[s] += sum_i w[i][j] in[i][8 g + s], i < n in order, for the thread's unit j and eight samples
-__device__ __forceinline__ void tile_dense(const float *w, const float *in, int n, int j, int g,
+// acc[s] += sum_i w[i stride] in[i ROW + s], i < n in order: one unit, eight samples
+template <int ROW>
+__device__ __forceinline__ void tile_dense(const float *w, int stride, const float *in, int n,
                                            float (&acc)[8]) {
+#pragma unroll 4
     for (int i = 0; i < n; ++i) {
-        const float c = w[i * kWRow + j];
-        const float4 a = *reinterpret_cast<const float4 *>(in + i * kRow + 8 * g);
-        const float4 b = *reinterpret_cast<const float4 *>(in + i * kRow + 8 * g + 4);
+        const float c = w[i * stride];
+        const float4 a = *reinterpret_cast<const float4 *>(in + i * ROW);
+        const float4 b = *reinterpret_cast<const float4 *>(in + i * ROW + 4);
         acc[0] = fmaf(a.x, c, acc[0]);
         acc[1] = fmaf(a.y, c, acc[1]);
         acc[2] = fmaf(a.z, c, acc[2]);
@@ -227,23 +240,23 @@ __device__ __forceinline__ void tile_dense(const float *w, const float *in, int 
         acc[7] = fmaf(b.w, c, acc[7]);
     }
 }
-__device__ __forceinline__ void put8(float *row, int g, const float (&v)[8]) {
-    *reinterpret_cast<float4 *>(row + 8 * g) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4 *>(row + 8 * g + 4) = make_float4(v[4], v[5], v[6], v[7]);
+__device__ __forceinline__ void put8(float *at, const float (&v)[8]) {
+    *reinterpret_cast<float4 *>(at) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4 *>(at + 4) = make_float4(v[4], v[5], v[6], v[7]);
 }
-// acc[a][b] += sum over the tile's samples of delta[j0 + 16 a] in[i0 + 16 b], samples in order
-__device__ __forceinline__ void tile_wgrad(const float *delta, const float *in, int j0, int i0,
-                                           float (&acc)[4][4]) {
+// acc[a][b] += sum_s z[8 a][s] in[16 b][s], bias[a] += sum_s z[8 a][s], s < ns in order
+__device__ __forceinline__ void chunk_wgrad(const float *z, const float *in, int ns,
+                                            float (&acc)[2][4], float (&bias)[2]) {
+    int s = 0;
 #pragma unroll 2
-    for (int s = 0; s < kTile; s += 4) {
-        float4 u[4], v[4];
+    for (; s + 4 <= ns; s += 4) {
+        float4 u[2], v[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            u[q] = *reinterpret_cast<const float4 *>(delta + (j0 + 16 * q) * kRow + s);
-            v[q] = *reinterpret_cast<const float4 *>(in + (i0 + 16 * q) * kRow + s);
-        }
+        for (int a = 0; a < 2; ++a) u[a] = *reinterpret_cast<const float4 *>(z + 8 * a * kCRow + s);
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int b = 0; b < 4; ++b) v[b] = *reinterpret_cast<const float4 *>(in + 16 * b * kCRow + s);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 acc[a][b] = fmaf(u[a].x, v[b].x, acc[a][b]);
@@ -251,191 +264,194 @@ __device__ __forceinline__ void tile_wgrad(const float *delta, const float *in, 
                 acc[a][b] = fmaf(u[a].z, v[b].z, acc[a][b]);
                 acc[a][b] = fmaf(u[a].w, v[b].w, acc[a][b]);
             }
+            bias[a] = bias[a] + u[a].x;
+            bias[a] = bias[a] + u[a].y;
+            bias[a] = bias[a] + u[a].z;
+            bias[a] = bias[a] + u[a].w;
+        }
     }
+    for (; s < ns; ++s)
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const float u = z[8 * a * kCRow + s];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(u, in[16 * b * kCRow + s], acc[a][b]);
+            bias[a] += u;
+        }
 }
 
-// Forward pass, loss and back-propagation of tiles b, b + gridDim.x, ... of 32 samples; the CTA's
-// gradients (the parameters' layout) and its share of the summed squared error go to
-// part[b (P + 1)].  Thread t: unit t % 64, samples 8 (t / 64) ... + 7 in the passes; a 4 x 4 block
-// of each weight gradient.  Training (stepc non-null): CTA 0 advances the Adam step counter, which
-// the update kernel after it reads.
-__global__ void __launch_bounds__(kThreads) mlp_tile_kernel(const float *p, int d, int H,
-                                                            const float *X, const float *t,
-                                                            long long n, float *part, int *stepc) {
+// Forward pass, back-propagation and weight-gradient sums of one chunk of kChunk samples by a
+// cluster of four CTAs: each takes a tile of 32 samples through the passes (thread t < 256: unit
+// t % 64, samples 8 (t / 64) ... + 7; warp 8: the output layer) and leaves its hidden states and
+// deltas in the shared memory of the CTAs that need them; then each sums the gradients of 16 units
+// over all 128 samples, so that every sum runs in the order of the general kernels above and the
+// results equal theirs bit for bit (training amplifies a last bit by orders of magnitude over 200
+// epochs).  The errors y - t go to err, the chunk's sums (the parameters' layout) to
+// part[chunk P].  Training (stepc non-null): CTA 0 advances the Adam step counter, which the update
+// kernel after it reads.  Bound by shared-memory latency: a chain of four dense passes, each a few
+// hundred cycles.
+__global__ void __cluster_dims__(kTiles, 1, 1) __launch_bounds__(kChunkThreads)
+    mlp_chunk_kernel(const float *p, int d, int H, const float *X, const float *t, long long n,
+                     float *err, float *part, int *stepc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TileSmem &M = *reinterpret_cast<TileSmem *>(smem_raw);
-    const int tid = threadIdx.x, j = tid & 63, g = tid >> 6;
+    ChunkSmem &M = *reinterpret_cast<ChunkSmem *>(smem_raw);
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), tid = threadIdx.x;
     const int P = H * d + H + H * H + H + H + 1;
     const float *W1 = p, *b1 = W1 + H * d, *W2 = b1 + H, *b2 = W2 + H * H, *W3 = b2 + H, *b3 = W3 + H;
+    const long long chunk = blockIdx.x / kTiles, s0 = chunk * kChunk;
+    const int ns = n - s0 < kChunk ? (int)(n - s0) : kChunk;  // samples of the chunk
     if (stepc && blockIdx.x == 0 && tid == 0) *stepc += 1;
-    for (int q = tid; q < kSmall * kWRow; q += kThreads) M.w1[q] = M.w2[q] = M.w2t[q] = 0.0f;
-    for (int q = tid; q < kSmall * kRow; q += kThreads) M.x[q] = 0.0f;
-    __syncthreads();
-    for (int q = tid; q < H * d; q += kThreads) M.w1[(q % d) * kWRow + q / d] = W1[q];
-    for (int q = tid; q < H * H; q += kThreads) {
-        const float w = W2[q];
-        M.w2[(q % H) * kWRow + q / H] = w;
-        M.w2t[(q / H) * kWRow + q % H] = w;
+    // (Units from H up and inputs from d up are never summed: their rows keep whatever is there.)
+    for (int q = tid; q < H * d; q += kChunkThreads) M.w1[(q % d) * kWRow + q / d] = W1[q];
+    for (int q = tid; q < H * H; q += kChunkThreads) M.w2[(q % H) * kWRow + q / H] = W2[q];
+    for (int q = tid; q < H; q += kChunkThreads) {
+        M.b1[q] = b1[q];
+        M.b2[q] = b2[q];
+        M.w3[q] = W3[q];
     }
-    if (tid < kSmall) {
-        M.b1[tid] = tid < H ? b1[tid] : 0.0f;
-        M.b2[tid] = tid < H ? b2[tid] : 0.0f;
-        M.w3[tid] = tid < H ? W3[tid] : 0.0f;
+    for (int q = tid; q < kChunk * d; q += kChunkThreads) {
+        const int s = q / d, i = q - s * d;
+        M.x[i * kCRow + s] = s < ns ? X[s0 * d + q] : 0.0f;
     }
-    const int j0 = tid >> 4, i0 = tid & 15;
-    float g1[4][4] = {}, g2[4][4] = {};  // gradients of W1 and W2
-    float gb1 = 0.0f, gb2 = 0.0f, gw3 = 0.0f, gb3 = 0.0f, loss = 0.0f;
-    const float bias3 = b3[0];
-    const long long tiles = (n + kTile - 1) / kTile;
-    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const long long s0 = tile * kTile;
-        const int ns = n - s0 < kTile ? (int)(n - s0) : kTile;
-        __syncthreads();  // the weights are there; the previous tile's rows are free
-        for (int q = tid; q < kTile * d; q += kThreads) {
-            const int s = q / d, i = q - s * d;
-            M.x[i * kRow + s] = s < ns ? X[s0 * d + q] : 0.0f;
-        }
-        __syncthreads();
-        float acc[8];
+    const bool unit = tid < kThreads;
+    const int j = tid & 63, g = (tid >> 6) & 3, lane = tid & 31;
+    const int col = kTile * rank + 8 * g;                  // the thread's samples in the chunk
+    const int own = (j % kUnits) * kCRow + col;            // and its place in the unit's CTA
+    cluster.sync();  // the weights and inputs are there; every CTA of the cluster runs
+    float acc[8];
+    if (unit) {
 #pragma unroll
         for (int s = 0; s < 8; ++s) acc[s] = M.b1[j];
-        tile_dense(M.w1, M.x, d, j, g, acc);
+        tile_dense<kCRow>(M.w1 + j, kWRow, M.x + col, d, acc);
 #pragma unroll
         for (int s = 0; s < 8; ++s) acc[s] = tanhf(acc[s]);
-        put8(M.h1 + j * kRow, g, acc);
-        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kTiles; ++r) put8(cluster.map_shared_rank(M.h1, r) + j * kCRow + col, acc);
+    }
+    __syncthreads();
+    if (unit) {
 #pragma unroll
         for (int s = 0; s < 8; ++s) acc[s] = M.b2[j];
-        tile_dense(M.w2, M.h1, H, j, g, acc);
+        tile_dense<kCRow>(M.w2 + j, kWRow, M.h1 + col, H, acc);
 #pragma unroll
         for (int s = 0; s < 8; ++s) acc[s] = tanhf(acc[s]);
-        put8(M.h2 + j * kRow, g, acc);
-        __syncthreads();
-        if (tid < kTile) {  // output and loss of one sample
-            float y = bias3;
-            for (int i = 0; i < H; ++i) y = fmaf(M.h2[i * kRow + tid], M.w3[i], y);
-            const float e = tid < ns ? y - t[s0 + tid] : 0.0f;
-            M.dy[tid] = 2.0f * e / (float)n;
-            loss = fmaf(e, e, loss);
-        }
-        __syncthreads();
-        {  // back through the output layer: h2 still in acc
-            float z[8];
-#pragma unroll
-            for (int s = 0; s < 8; ++s)
-                z[s] = fmaf(M.dy[8 * g + s], M.w3[j], 0.0f) * (1.0f - acc[s] * acc[s]);
-            put8(M.z2 + j * kRow, g, z);
-        }
-        __syncthreads();
-        {  // back through the second layer
-            float z[8] = {};
-            tile_dense(M.w2t, M.z2, H, j, g, z);
-            const float4 a = *reinterpret_cast<const float4 *>(M.h1 + j * kRow + 8 * g);
-            const float4 b = *reinterpret_cast<const float4 *>(M.h1 + j * kRow + 8 * g + 4);
-            const float h[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-            for (int s = 0; s < 8; ++s) z[s] = z[s] * (1.0f - h[s] * h[s]);
-            put8(M.z1 + j * kRow, g, z);
-        }
-        __syncthreads();
-        tile_wgrad(M.z1, M.x, j0, i0, g1);
-        tile_wgrad(M.z2, M.h1, j0, i0, g2);
-        if (g == 0)
-            for (int s = 0; s < kTile; ++s) gb1 += M.z1[j * kRow + s];
-        if (g == 1)
-            for (int s = 0; s < kTile; ++s) gb2 += M.z2[j * kRow + s];
-        if (g == 2)
-            for (int s = 0; s < kTile; ++s) gw3 = fmaf(M.dy[s], M.h2[j * kRow + s], gw3);
-        if (tid == 255)
-            for (int s = 0; s < kTile; ++s) gb3 += M.dy[s];
+        put8(M.h2 + j * kRow + 8 * g, acc);
+        put8(cluster.map_shared_rank(M.h2c, j / kUnits) + own, acc);
     }
-    float *out = part + (long long)blockIdx.x * (P + 1);
-    float *o1 = out + H * d, *o2 = o1 + H, *o3 = o2 + H * H, *o4 = o3 + H, *o5 = o4 + H;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int r = j0 + 16 * a, c = i0 + 16 * b;
-            if (r < H && c < d) out[r * d + c] = g1[a][b];
-            if (r < H && c < H) o2[r * H + c] = g2[a][b];
-        }
-    if (j < H) {
-        if (g == 0) o1[j] = gb1;
-        if (g == 1) o3[j] = gb2;
-        if (g == 2) o4[j] = gw3;
-    }
-    if (tid == 255) o5[0] = gb3;
-    if (tid < kTile) M.loss[tid] = loss;
     __syncthreads();
-    if (tid == 0) {
+    if (!unit) {  // output and error of one sample
+        float y = b3[0];
+#pragma unroll 8
+        for (int i = 0; i < H; ++i) y = fmaf(M.h2[i * kRow + lane], M.w3[i], y);
+        const int s = kTile * rank + lane;
         float e = 0.0f;
-        for (int s = 0; s < kTile; ++s) e += M.loss[s];
-        out[P] = e;
+        if (s < ns) {
+            e = y - t[s0 + s];
+            err[s0 + s] = e;
+        }
+        const float dy = 2.0f * e / (float)n;
+#pragma unroll
+        for (int r = 0; r < kTiles; ++r) cluster.map_shared_rank(M.dy, r)[s] = dy;
+    }
+    __syncthreads();
+    if (unit) {  // back through the output layer: h2 still in acc
+        float z[8];
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+            z[s] = fmaf(M.dy[col + s], M.w3[j], 0.0f) * (1.0f - acc[s] * acc[s]);
+        put8(M.z2 + j * kRow + 8 * g, z);
+        put8(cluster.map_shared_rank(M.z2c, j / kUnits) + own, z);
+    }
+    __syncthreads();
+    if (unit) {  // back through the second layer
+        float z[8] = {};
+        tile_dense<kRow>(M.w2 + j * kWRow, 1, M.z2 + 8 * g, H, z);
+        const float *h = M.h1 + j * kCRow + col;
+#pragma unroll
+        for (int s = 0; s < 8; ++s) z[s] = z[s] * (1.0f - h[s] * h[s]);
+        put8(cluster.map_shared_rank(M.z1c, j / kUnits) + own, z);
+    }
+    cluster.sync();  // the chunk's states and deltas are there
+    float *out = part + chunk * P;
+    float *o1 = out + H * d, *o2 = o1 + H, *o3 = o2 + H * H, *o4 = o3 + H, *o5 = o4 + H;
+    if (unit) {  // threads 0-127: W1 and b1; 128-255: W2 and b2
+        const int u = tid & 127, j0 = u >> 4, i0 = u & 15;
+        const bool first = tid < 128;
+        const int cols = first ? d : H;
+        float gw[2][4] = {}, gb[2] = {};
+        chunk_wgrad((first ? M.z1c : M.z2c) + j0 * kCRow, (first ? M.x : M.h1) + i0 * kCRow, ns, gw,
+                    gb);
+        float *ow = first ? out : o2, *ob = first ? o1 : o3;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const int r = kUnits * rank + j0 + 8 * a;
+            if (r >= H) continue;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                if (i0 + 16 * b < cols) ow[r * cols + i0 + 16 * b] = gw[a][b];
+            if (i0 == 0) ob[r] = gb[a];
+        }
+    } else if (lane <= kUnits) {  // W3; b3
+        const int r = kUnits * rank + lane;
+        float sum = 0.0f;
+        if (lane < kUnits) {
+#pragma unroll 8
+            for (int s = 0; s < ns; ++s) sum = fmaf(M.dy[s], M.h2c[lane * kCRow + s], sum);
+            if (r < H) o4[r] = sum;
+        } else if (rank == 0) {
+#pragma unroll 8
+            for (int s = 0; s < ns; ++s) sum += M.dy[s];
+            o5[0] = sum;
+        }
     }
 }
 
-constexpr int kUpdateParams = 32;  // parameters of an update CTA, eight threads each
-
-// grad = the sum of the tile CTAs' gradients, eight runs of CTAs in parallel, the runs in order;
-// then, training (stepc non-null), the Adam update of adam_kernel_dev, with what rounding a
-// parameter to FP32 leaves out carried to its next update (rest; TwoSum): an update of about lr is
-// 1e-3 of a parameter, and without that 200 updates' roundings are most of the result's error.
-// The thread of index P sums the losses.
+// grad = the chunks' sums added in chunk order; then, training (stepc non-null), the Adam update.
+// The last CTA adds up the loss as mse_kernel does.
 __global__ void __launch_bounds__(kThreads)
-    mlp_update_kernel(const float *part, int ctas, int P, long long n, float *grad, float *loss_out,
-                      float *p, float *m, float *v, float *rest, float lr, float b1, float b2,
-                      float eps, const int *stepc, int step0, float *hist) {
-    __shared__ float run[8][kUpdateParams];
-    const int q = threadIdx.x & (kUpdateParams - 1), r = threadIdx.x / kUpdateParams;
-    const int i = blockIdx.x * kUpdateParams + q;
-    const int c0 = ctas * r / 8, c1 = ctas * (r + 1) / 8;
-    float acc = 0.0f;
-    if (i <= P) {
+    mlp_update_kernel(const float *part, const float *err, int chunks, int P, long long n,
+                      float *grad, float *loss_out, float *p, float *m, float *v, float lr,
+                      float b1, float b2, float eps, const int *stepc, int step0, float *hist) {
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ float s[kThreads];
+        float acc = 0.0f;
 #pragma unroll 8
-        for (int c = c0; c < c1; ++c) acc += part[(long long)c * (P + 1) + i];
-    }
-    run[r][q] = acc;
-    __syncthreads();
-    if (r != 0 || i > P) return;
-#pragma unroll
-    for (int k = 1; k < 8; ++k) acc += run[k][q];
-    if (i == P) {
-        const float loss = acc / (float)n;
-        *loss_out = loss;
-        if (stepc && hist) hist[*stepc - 1 - step0] = loss;
+        for (long long i = threadIdx.x; i < n; i += kThreads) acc = fmaf(err[i], err[i], acc);
+        const float sum = block_sum(s, acc);
+        if (threadIdx.x == 0) {
+            *loss_out = sum / (float)n;
+            if (stepc && hist) hist[*stepc - 1 - step0] = sum / (float)n;
+        }
         return;
     }
+    const int i = blockIdx.x * kThreads + threadIdx.x;
+    if (i >= P) return;
+    float acc = 0.0f;
+#pragma unroll 16
+    for (int c = 0; c < chunks; ++c) acc += part[(long long)c * P + i];
     grad[i] = acc;
-    if (!stepc) return;
-    const float t = (float)*stepc;
-    const float k1 = 1.0f - powf(b1, t), k2 = 1.0f - powf(b2, t);
-    const float mi = b1 * m[i] + (1.0f - b1) * acc;
-    const float vi = b2 * v[i] + (1.0f - b2) * acc * acc;
-    m[i] = mi;
-    v[i] = vi;
-    const float q0 = p[i], y = __fadd_rn(rest[i], -(lr * (mi / k1) / (sqrtf(vi / k2) + eps)));
-    const float q1 = __fadd_rn(q0, y), back = __fadd_rn(q1, -q0);
-    rest[i] = __fadd_rn(__fadd_rn(q0, -__fadd_rn(q1, -back)), __fadd_rn(y, -back));
-    p[i] = q1;
+    if (stepc) adam_step(p, m, v, i, acc, lr, b1, b2, eps, (float)*stepc);
 }
 
 // One small-network epoch (or, with m null, the gradient alone).
 cudaError_t small_epoch(float *p, float *m, float *v, int d, int H, const float *X, const float *t,
                         long long n, float *ws, const Sizes &S, float lr, int *stepc, int step0,
                         float *hist, cudaStream_t st) {
-    const int ctas = (int)tile_ctas(n), P = (int)S.P;
-    float *part = ws + S.part;
-    mlp_tile_kernel<<<ctas, kThreads, sizeof(TileSmem), st>>>(p, d, H, X, t, n, part, stepc);
-    mlp_update_kernel<<<(P + 1 + kUpdateParams - 1) / kUpdateParams, kThreads, 0, st>>>(
-        part, ctas, P, n, ws + S.grad, ws + S.loss, p, m, v, ws + S.rest, lr, 0.9f, 0.999f, 1e-8f,
-        stepc, step0, hist);
+    const int chunks = (int)((n + kChunk - 1) / kChunk), P = (int)S.P;
+    float *part = ws + S.part, *err = ws + S.y;
+    mlp_chunk_kernel<<<chunks * kTiles, kChunkThreads, sizeof(ChunkSmem), st>>>(p, d, H, X, t, n,
+                                                                                err, part, stepc);
+    mlp_update_kernel<<<(P + kThreads - 1) / kThreads + 1, kThreads, 0, st>>>(
+        part, err, chunks, P, n, ws + S.grad, ws + S.loss, p, m, v, lr, 0.9f, 0.999f, 1e-8f, stepc,
+        step0, hist);
     return cudaGetLastError();
 }
 cudaError_t small_prepare() {
     static hydro::PerDevice attribute;
     return attribute.once([] {
-        return cudaFuncSetAttribute(mlp_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sizeof(TileSmem));
+        return cudaFuncSetAttribute(mlp_chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sizeof(ChunkSmem));
     });
 }
 
@@ -569,7 +585,6 @@ int hydro_mlp_train(float *params, float *m, float *v, int32_t d, int32_t hidden
     cudaError_t e = cudaGetLastError();
     if (small_net(d, hidden)) {  // two launches an epoch: the GPU, not the launches, sets the pace
         if (e == cudaSuccess) e = small_prepare();
-        if (e == cudaSuccess) e = cudaMemsetAsync(ws + S.rest, 0, sizeof(float) * (size_t)S.P, st);
         for (int k = 0; k < epochs && e == cudaSuccess; ++k)
             e = small_epoch(params, m, v, d, hidden, X, t, n, ws, S, lr, stepc, step0, loss_out, st);
         return e == cudaSuccess ? HYDRO_OK : hydro::record_cuda_error(e, "hydro_mlp_train");
