@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(kWaveThreads)
 constexpr int kClusterMax = 16;        // CTAs of the cluster (beyond the portable 8)
 constexpr int kClusterThreads = 256;
 constexpr int kClusterPer = 4;         // cells of a thread at most
+constexpr int kClusterSteps = 4096;    // steps of a launch
 constexpr int kClusterCells = kClusterMax * kClusterThreads * kClusterPer;
 
 __device__ __forceinline__ void cluster_sync() {
@@ -418,8 +419,9 @@ WaveLayout wave_layout(long long n, int prec, int n_steps) {
     L.g_off = align_up((size_t)n * esz);
     L.part_off = L.g_off + align_up((size_t)n * esz);
     size_t parts = (size_t)L.nblocks;
-    if (n <= kClusterCells && (size_t)n_steps * kClusterMax > parts)
-        parts = (size_t)n_steps * kClusterMax;  // a sum per CTA of the cluster and step
+    const size_t chunk = (size_t)(n_steps < kClusterSteps ? n_steps : kClusterSteps);
+    if (n <= kClusterCells && chunk * kClusterMax > parts)
+        parts = chunk * kClusterMax;  // a sum per CTA of the cluster and step of one launch
     L.e_off = L.part_off + align_up(sizeof(double) * parts);
     L.total = L.e_off + align_up(sizeof(double) * (size_t)(n_steps > 0 ? n_steps : 1));
     return L;
@@ -483,15 +485,19 @@ int wave_run_t(long long n, double c, double length, double dt, T *f, T *g, int 
         cudaLaunchAttribute attr;
         if (cluster_config<T>(n, &cfg, &attr, st)) {
             const int C = (int)cfg.gridDim.x, per = (int)((n + C - 1) / C);
-            cudaError_t e = cudaLaunchKernelEx(&cfg, wave_cluster_kernel<T>, f, g, (int)n, per, n_steps,
-                                               T(dt), k, k1, k2, part);
-            if (e == cudaSuccess && energy_out) {
-                wave_cluster_energy_kernel<<<(n_steps + 255) / 256, 256, 0, st>>>(part, C, n_steps, energy);
-                e = cudaGetLastError();
-                if (e == cudaSuccess)
-                    e = cudaMemcpyAsync(energy_out, energy, sizeof(double) * (size_t)n_steps,
-                                        cudaMemcpyDeviceToHost, st);
+            cudaError_t e = cudaSuccess;
+            for (int s0 = 0; s0 < n_steps && e == cudaSuccess; s0 += kClusterSteps) {
+                const int m = n_steps - s0 < kClusterSteps ? n_steps - s0 : kClusterSteps;
+                e = cudaLaunchKernelEx(&cfg, wave_cluster_kernel<T>, f, g, (int)n, per, m, T(dt), k,
+                                       k1, k2, part);
+                if (e == cudaSuccess && energy_out) {
+                    wave_cluster_energy_kernel<<<(m + 255) / 256, 256, 0, st>>>(part, C, m, energy + s0);
+                    e = cudaGetLastError();
+                }
             }
+            if (e == cudaSuccess && energy_out)
+                e = cudaMemcpyAsync(energy_out, energy, sizeof(double) * (size_t)n_steps,
+                                    cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             return e == cudaSuccess ? HYDRO_OK : hydro::record_cuda_error(e, "hydro_wave_run");
         }
