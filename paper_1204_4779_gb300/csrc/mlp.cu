@@ -16,7 +16,7 @@
 // the shared memory of a thread-block cluster and leaves the chunk's weight gradients;
 // mlp_update_kernel sums them in chunk order and applies Adam.  The thirteen launches of the
 // general kernels took 174 us an epoch (4200 records, 35 inputs, width 64), most of it in gathers
-// and launches; the two take 27, with equal bits.  The general kernels serve wider networks.
+// and launches; the two take 23.4, with equal bits.  The general kernels serve wider networks.
 //
 // There training replays captured epochs: the Adam step number lives in the workspace (the loss
 // kernel advances it, the Adam kernel derives its bias corrections from it), so one epoch's
@@ -45,7 +45,8 @@ constexpr int kSmall = 64;                // most inputs and hidden units of the
 constexpr int kTile = 32;                 // samples of a CTA's tile
 constexpr int kTiles = kChunk / kTile;    // CTAs of a cluster
 constexpr int kUnits = kSmall / kTiles;   // units whose gradients a CTA sums
-constexpr int kChunkThreads = kThreads + 32;
+constexpr int kPass = 512;                // threads of the passes: a unit, four samples each
+constexpr int kChunkThreads = kPass + 32;
 constexpr int kRow = kTile + 4;           // floats of a shared row of a tile,
 constexpr int kCRow = kChunk + 4;         // of a chunk (rows on distinct banks)
 constexpr int kWRow = kSmall + 1;         // and of a weight matrix (either index conflict-free)
@@ -221,44 +222,47 @@ struct ChunkSmem {
     float dy[kChunk];
 };
 
-// acc[s] += sum_i w[i stride] in[i ROW + s], i < n in order: one unit, eight samples
+// Asynchronous copy of one float to shared memory; zero where !valid (`from` is readable anyway)
+__device__ __forceinline__ void copy4(float *to, const float *from, bool valid = true) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(to)),
+                 "l"(from), "r"(valid ? 4 : 0)
+                 : "memory");
+}
+
+// acc[s] += sum_i w[i stride] in[i ROW + s], i < n in order: one unit, four samples
 template <int ROW>
 __device__ __forceinline__ void tile_dense(const float *w, int stride, const float *in, int n,
-                                           float (&acc)[8]) {
-#pragma unroll 4
+                                           float (&acc)[4]) {
+#pragma unroll 8
     for (int i = 0; i < n; ++i) {
         const float c = w[i * stride];
         const float4 a = *reinterpret_cast<const float4 *>(in + i * ROW);
-        const float4 b = *reinterpret_cast<const float4 *>(in + i * ROW + 4);
         acc[0] = fmaf(a.x, c, acc[0]);
         acc[1] = fmaf(a.y, c, acc[1]);
         acc[2] = fmaf(a.z, c, acc[2]);
         acc[3] = fmaf(a.w, c, acc[3]);
-        acc[4] = fmaf(b.x, c, acc[4]);
-        acc[5] = fmaf(b.y, c, acc[5]);
-        acc[6] = fmaf(b.z, c, acc[6]);
-        acc[7] = fmaf(b.w, c, acc[7]);
     }
 }
-__device__ __forceinline__ void put8(float *at, const float (&v)[8]) {
+__device__ __forceinline__ void put4(float *at, const float (&v)[4]) {
     *reinterpret_cast<float4 *>(at) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4 *>(at + 4) = make_float4(v[4], v[5], v[6], v[7]);
 }
 // acc[a][b] += sum_s z[8 a][s] in[16 b][s], bias[a] += sum_s z[8 a][s], s < ns in order
 __device__ __forceinline__ void chunk_wgrad(const float *z, const float *in, int ns,
-                                            float (&acc)[2][4], float (&bias)[2]) {
+                                            float (&acc)[2][2], float (&bias)[2]) {
     int s = 0;
-#pragma unroll 2
+#pragma unroll 4
     for (; s + 4 <= ns; s += 4) {
-        float4 u[2], v[4];
+        float4 u[2], v[2];
 #pragma unroll
-        for (int a = 0; a < 2; ++a) u[a] = *reinterpret_cast<const float4 *>(z + 8 * a * kCRow + s);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) v[b] = *reinterpret_cast<const float4 *>(in + 16 * b * kCRow + s);
+        for (int a = 0; a < 2; ++a) {
+            u[a] = *reinterpret_cast<const float4 *>(z + 8 * a * kCRow + s);
+            v[a] = *reinterpret_cast<const float4 *>(in + 16 * a * kCRow + s);
+        }
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
+            for (int b = 0; b < 2; ++b) {
                 acc[a][b] = fmaf(u[a].x, v[b].x, acc[a][b]);
                 acc[a][b] = fmaf(u[a].y, v[b].y, acc[a][b]);
                 acc[a][b] = fmaf(u[a].z, v[b].z, acc[a][b]);
@@ -275,21 +279,21 @@ __device__ __forceinline__ void chunk_wgrad(const float *z, const float *in, int
         for (int a = 0; a < 2; ++a) {
             const float u = z[8 * a * kCRow + s];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(u, in[16 * b * kCRow + s], acc[a][b]);
+            for (int b = 0; b < 2; ++b) acc[a][b] = fmaf(u, in[16 * b * kCRow + s], acc[a][b]);
             bias[a] += u;
         }
 }
 
 // Forward pass, back-propagation and weight-gradient sums of one chunk of kChunk samples by a
-// cluster of four CTAs: each takes a tile of 32 samples through the passes (thread t < 256: unit
-// t % 64, samples 8 (t / 64) ... + 7; warp 8: the output layer) and leaves its hidden states and
+// cluster of four CTAs: each takes a tile of 32 samples through the passes (thread t < 512: unit
+// t % 64, samples 4 (t / 64) ... + 3; warp 16: the output layer) and leaves its hidden states and
 // deltas in the shared memory of the CTAs that need them; then each sums the gradients of 16 units
 // over all 128 samples, so that every sum runs in the order of the general kernels above and the
 // results equal theirs bit for bit (training amplifies a last bit by orders of magnitude over 200
 // epochs).  The errors y - t go to err, the chunk's sums (the parameters' layout) to
 // part[chunk P].  Training (stepc non-null): CTA 0 advances the Adam step counter, which the update
-// kernel after it reads.  Bound by shared-memory latency: a chain of four dense passes, each a few
-// hundred cycles.
+// kernel after it reads.  Bound by shared-memory accesses (LSU wavefronts 48 % busy) along a
+// chain of five dependent passes; 17.6 us of the epoch under a profiler with cold caches.
 __global__ void __cluster_dims__(kTiles, 1, 1) __launch_bounds__(kChunkThreads)
     mlp_chunk_kernel(const float *p, int d, int H, const float *X, const float *t, long long n,
                      float *err, float *part, int *stepc) {
@@ -303,41 +307,52 @@ __global__ void __cluster_dims__(kTiles, 1, 1) __launch_bounds__(kChunkThreads)
     const int ns = n - s0 < kChunk ? (int)(n - s0) : kChunk;  // samples of the chunk
     if (stepc && blockIdx.x == 0 && tid == 0) *stepc += 1;
     // (Units from H up and inputs from d up are never summed: their rows keep whatever is there.)
-    for (int q = tid; q < H * d; q += kChunkThreads) M.w1[(q % d) * kWRow + q / d] = W1[q];
-    for (int q = tid; q < H * H; q += kChunkThreads) M.w2[(q % H) * kWRow + q / H] = W2[q];
-    for (int q = tid; q < H; q += kChunkThreads) {
-        M.b1[q] = b1[q];
-        M.b2[q] = b2[q];
-        M.w3[q] = W3[q];
+    // Asynchronous copies, a warp per row: plain loads in a loop wait for one another (an epoch of
+    // 27.5 us instead of 25.4 with them).
+    const int lane = tid & 31, warp = tid >> 5;
+    for (int r = warp; r < kChunk; r += kChunkThreads / 32)
+        for (int i = lane; i < d; i += 32)
+            copy4(&M.x[i * kCRow + r], X + (s0 + (r < ns ? r : 0)) * d + i, r < ns);
+    for (int r = warp; r < H; r += kChunkThreads / 32) {
+        for (int i = lane; i < d; i += 32) copy4(&M.w1[i * kWRow + r], W1 + r * d + i);
+        for (int i = lane; i < H; i += 32) copy4(&M.w2[i * kWRow + r], W2 + r * H + i);
     }
-    for (int q = tid; q < kChunk * d; q += kChunkThreads) {
-        const int s = q / d, i = q - s * d;
-        M.x[i * kCRow + s] = s < ns ? X[s0 * d + q] : 0.0f;
+    if (tid < H) {
+        copy4(&M.b1[tid], b1 + tid);
+        copy4(&M.b2[tid], b2 + tid);
+        copy4(&M.w3[tid], W3 + tid);
     }
-    const bool unit = tid < kThreads;
-    const int j = tid & 63, g = (tid >> 6) & 3, lane = tid & 31;
-    const int col = kTile * rank + 8 * g;                  // the thread's samples in the chunk
-    const int own = (j % kUnits) * kCRow + col;            // and its place in the unit's CTA
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+    const bool unit = tid < kPass;
+    const int j = tid & 63, g = (tid >> 6) & 7;
+    const int col = kTile * rank + 4 * g;  // the thread's samples in the chunk
+    // What other CTAs need goes to them from shared memory, eight lanes per row of 128 B: stores of
+    // a unit per lane are 32 separate packets each (an epoch of 25.4 us instead of 23.4).
+    const int row = tid >> 3, at = 4 * (tid & 7), seat = (row % kUnits) * kCRow + kTile * rank + at;
+    const int seat_rank = (row / kUnits) % kTiles;
     cluster.sync();  // the weights and inputs are there; every CTA of the cluster runs
-    float acc[8];
+    float acc[4];
     if (unit) {
 #pragma unroll
-        for (int s = 0; s < 8; ++s) acc[s] = M.b1[j];
+        for (int s = 0; s < 4; ++s) acc[s] = M.b1[j];
         tile_dense<kCRow>(M.w1 + j, kWRow, M.x + col, d, acc);
 #pragma unroll
-        for (int s = 0; s < 8; ++s) acc[s] = tanhf(acc[s]);
-#pragma unroll
-        for (int r = 0; r < kTiles; ++r) put8(cluster.map_shared_rank(M.h1, r) + j * kCRow + col, acc);
+        for (int s = 0; s < 4; ++s) acc[s] = tanhf(acc[s]);
+        put4(M.h1 + j * kCRow + col, acc);
     }
     __syncthreads();
     if (unit) {
+        const int o = row * kCRow + kTile * rank + at;
+        const float4 h = *reinterpret_cast<const float4 *>(M.h1 + o);
 #pragma unroll
-        for (int s = 0; s < 8; ++s) acc[s] = M.b2[j];
+        for (int r = 1; r < kTiles; ++r)
+            *reinterpret_cast<float4 *>(cluster.map_shared_rank(M.h1, (rank + r) % kTiles) + o) = h;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) acc[s] = M.b2[j];
         tile_dense<kCRow>(M.w2 + j, kWRow, M.h1 + col, H, acc);
 #pragma unroll
-        for (int s = 0; s < 8; ++s) acc[s] = tanhf(acc[s]);
-        put8(M.h2 + j * kRow + 8 * g, acc);
-        put8(cluster.map_shared_rank(M.h2c, j / kUnits) + own, acc);
+        for (int s = 0; s < 4; ++s) acc[s] = tanhf(acc[s]);
+        put4(M.h2 + j * kRow + 4 * g, acc);
     }
     __syncthreads();
     if (!unit) {  // output and error of one sample
@@ -356,41 +371,50 @@ __global__ void __cluster_dims__(kTiles, 1, 1) __launch_bounds__(kChunkThreads)
     }
     __syncthreads();
     if (unit) {  // back through the output layer: h2 still in acc
-        float z[8];
+        *reinterpret_cast<float4 *>(cluster.map_shared_rank(M.h2c, seat_rank) + seat) =
+            *reinterpret_cast<const float4 *>(M.h2 + row * kRow + at);
+        float z[4];
 #pragma unroll
-        for (int s = 0; s < 8; ++s)
+        for (int s = 0; s < 4; ++s)
             z[s] = fmaf(M.dy[col + s], M.w3[j], 0.0f) * (1.0f - acc[s] * acc[s]);
-        put8(M.z2 + j * kRow + 8 * g, z);
-        put8(cluster.map_shared_rank(M.z2c, j / kUnits) + own, z);
+        put4(M.z2 + j * kRow + 4 * g, z);
     }
     __syncthreads();
     if (unit) {  // back through the second layer
-        float z[8] = {};
-        tile_dense<kRow>(M.w2 + j * kWRow, 1, M.z2 + 8 * g, H, z);
+        *reinterpret_cast<float4 *>(cluster.map_shared_rank(M.z2c, seat_rank) + seat) =
+            *reinterpret_cast<const float4 *>(M.z2 + row * kRow + at);
+        float z[4] = {};
+        tile_dense<kRow>(M.w2 + j * kWRow, 1, M.z2 + 4 * g, H, z);
         const float *h = M.h1 + j * kCRow + col;
 #pragma unroll
-        for (int s = 0; s < 8; ++s) z[s] = z[s] * (1.0f - h[s] * h[s]);
-        put8(cluster.map_shared_rank(M.z1c, j / kUnits) + own, z);
+        for (int s = 0; s < 4; ++s) z[s] = z[s] * (1.0f - h[s] * h[s]);
+        put4(M.h2 + j * kRow + 4 * g, z);  // (h2 is no longer read)
     }
+    __syncthreads();
+    if (unit)
+        *reinterpret_cast<float4 *>(cluster.map_shared_rank(M.z1c, seat_rank) + seat) =
+            *reinterpret_cast<const float4 *>(M.h2 + row * kRow + at);
     cluster.sync();  // the chunk's states and deltas are there
     float *out = part + chunk * P;
     float *o1 = out + H * d, *o2 = o1 + H, *o3 = o2 + H * H, *o4 = o3 + H, *o5 = o4 + H;
-    if (unit) {  // threads 0-127: W1 and b1; 128-255: W2 and b2
-        const int u = tid & 127, j0 = u >> 4, i0 = u & 15;
-        const bool first = tid < 128;
+    if (unit) {  // threads 0-255: W1 and b1; 256-511: W2 and b2; two units, two inputs each
+        const bool first = tid < kPass / 2;
         const int cols = first ? d : H;
-        float gw[2][4] = {}, gb[2] = {};
-        chunk_wgrad((first ? M.z1c : M.z2c) + j0 * kCRow, (first ? M.x : M.h1) + i0 * kCRow, ns, gw,
-                    gb);
-        float *ow = first ? out : o2, *ob = first ? o1 : o3;
+        const int j0 = (tid >> 4) & 7, i0 = (tid & 15) + (tid & 128) / 4;
+        if (i0 < cols) {
+            float gw[2][2] = {}, gb[2] = {};
+            chunk_wgrad((first ? M.z1c : M.z2c) + j0 * kCRow, (first ? M.x : M.h1) + i0 * kCRow, ns,
+                        gw, gb);
+            float *ow = first ? out : o2, *ob = first ? o1 : o3;
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            const int r = kUnits * rank + j0 + 8 * a;
-            if (r >= H) continue;
+            for (int a = 0; a < 2; ++a) {
+                const int r = kUnits * rank + j0 + 8 * a;
+                if (r >= H) continue;
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
-                if (i0 + 16 * b < cols) ow[r * cols + i0 + 16 * b] = gw[a][b];
-            if (i0 == 0) ob[r] = gb[a];
+                for (int b = 0; b < 2; ++b)
+                    if (i0 + 16 * b < cols) ow[r * cols + i0 + 16 * b] = gw[a][b];
+                if (i0 == 0) ob[r] = gb[a];
+            }
         }
     } else if (lane <= kUnits) {  // W3; b3
         const int r = kUnits * rank + lane;
@@ -428,7 +452,7 @@ __global__ void __launch_bounds__(kThreads)
     const int i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= P) return;
     float acc = 0.0f;
-#pragma unroll 16
+#pragma unroll 32
     for (int c = 0; c < chunks; ++c) acc += part[(long long)c * P + i];
     grad[i] = acc;
     if (stepc) adam_step(p, m, v, i, acc, lr, b1, b2, eps, (float)*stepc);
