@@ -43,9 +43,10 @@ def _peaks():
 
 # the sources each committed ncu record depends on: a record whose digest differs was taken on
 # other kernel code and is not used
-STAGE_SOURCES = ("hydro_device.cuh", "stage_kernel.cuh", "stage_launch.cuh", "stage_f32_d3.cu",
-                 "stage_f32_d3b.cu")
-BATCH_SOURCES = ("hydro_device.cuh", "stage_kernel.cuh", "batch_kernel.cuh", "batch_f32.cu")
+STAGE_SOURCES = ("hydro_device.cuh", "pair_device.cuh", "row_kernel.cuh", "strip3_kernel.cuh",
+                 "stage_strip3.cu")
+BATCH_SOURCES = ("hydro_device.cuh", "pair_device.cuh", "row_kernel.cuh", "batch_kernel.cuh",
+                 "batch_f32.cu")
 
 
 def _kernel_digest(sources=STAGE_SOURCES) -> str:

@@ -137,7 +137,9 @@ typedef struct {
  * Strip kernels: the FP32 row tiles of dim 2 and, in dim 3, the FP32 tile 16 x 8 with look-ahead
  * staging and nothing manifest run kernels whose warps own strips of 64 columns, two cells per
  * lane, and march with everything in registers.  Of a row tile's width they take one warp per 64
- * columns; staging and occupancy do not apply to them.  Grids of dim 1 of 32 to 2048 cells with
+ * columns; staging and occupancy do not apply to them.  The FP64 tile 32 x 8 of dim 2 runs strips
+ * of 32 columns, one cell per lane, with periodic and outflow boundaries, and unless the variant
+ * names a split reduces dt in stage 2 (reported: the tile's default, 1).  Grids of dim 1 of 32 to 2048 cells with
  * periodic or outflow ends run whole chunks of steps in one launch, whatever the variant.
  * Library defaults (measured on GB300): dim 3 FP32 tile 16 x 8 (march from the grid size: 96
  * at 512^3), FP64 32 x 8, march 64; dim 2 FP32 row tile 256 x 1 (march from the grid size: 16
