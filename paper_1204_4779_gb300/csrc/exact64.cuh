@@ -16,10 +16,19 @@
 //  * square roots by the coupled iteration for sqrt and 1 / (2 sqrt) (Goldschmidt's) from the
 //    FP32 reciprocal root, closed by the same exact-remainder step: six operations against nine
 //    and a half.
-// The reciprocal is not always the correctly rounded one that Markstein's proof asks for (its
-// error before rounding is 2^-66): a quotient can miss only where it lies within about 2^-51 ulp
-// of a midpoint, a root within 2^-34 ulp.  Operands outside the range where no step under- or
-// overflows (exponents of +-400, or zero numerators) are the caller's to send to the plain
+//
+// Reciprocals and roots end in an integer comparison that settles the last place: the FP64 value
+// is within an ulp, so the exact integer remainder (B Y against a power of two for the
+// reciprocal, A 2^k - Z^2 for the root) fits 64 bits and says whether the value, or which
+// neighbour of it, is the correctly rounded one.  A quotient by a correctly rounded reciprocal is
+// correctly rounded for every divisor (Markstein's theorem), so these are the IEEE results, not
+// only nearly always: without the comparison roots within 2^-34 ulp of the middle of two doubles
+// came out an ulp off, and so did quotients next to it by divisors just below a power of two.
+// The integer instructions are ones the FP64 pipe's schedulers have to spare: 1024^2 stays at
+// 27.4 ms for 20 steps (the reciprocal's last place by a Newton step under a branch instead:
+// 28.2 ms); one warp alone waits for them (1024 cells, 1126 steps: 15.4 -> 15.7 ms).
+// Operands outside the range where no step under- or overflows (exponents of +-400, or zero
+// numerators other than a momentum or the numerator of S*) are the caller's to send to the plain
 // operations.
 #pragma once
 
@@ -56,14 +65,20 @@ struct Fma64 {
     __device__ __forceinline__ double add(double a, double b) const { return fma(a, one, b); }
     __device__ __forceinline__ double sub(double a, double b) const { return fma(-b, one, a); }
     __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, mzero); }
-    // a / b with y = recip64(b)
+    // a / b with y = recip64(b); a zero numerator (of a positive divisor) keeps its sign: the
+    // remainder's zero is subtracted, which leaves -0 as it is
     __device__ __forceinline__ double div(double a, double b, double y) const {
+        const double q = mul(a, y);
+        return fma(-fma(b, q, -a), y, q);
+    }
+    // the same where b < 0: there the remainder's zero has to be added
+    __device__ __forceinline__ double div_by_negative(double a, double b, double y) const {
         const double q = mul(a, y);
         return fma(fma(-b, q, a), y, q);
     }
 };
 
-// 1 / b within an ulp, b in range.
+// 1 / b, correctly rounded, b in range.
 __device__ __forceinline__ double recip64(double b) {
     const int hi = __double2hiint(b), lo = __double2loint(b);
     const float m = __int_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffff) | 0x3f800000);
@@ -74,7 +89,13 @@ __device__ __forceinline__ double recip64(double b) {
     const int h = ((rb >> 3) + ((2 * 1023 - 127 - e) << 20)) | (hi & (int)0x80000000);
     const double y = __hiloint2double(h, rb << 29);
     const double d = fma(-b, y, 1.0);
-    return fma(y, fma(d, d, d), y);
+    const long long z = __double_as_longlong(fma(y, fma(d, d, d), y));
+    // B Y = 2^104 or 2^105 minus the remainder, whose low 64 bits are all of it; Y is the rounded
+    // reciprocal if and only if |remainder| <= B / 2
+    const unsigned long long B = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)lo;
+    const unsigned long long Y = ((unsigned long long)z & 0xfffffffffffffull) | 0x10000000000000ull;
+    const long long R = (long long)(0ull - 2ull * (B * Y));
+    return __longlong_as_double(z + (R > (long long)B) - (R < -(long long)B));
 }
 
 // sqrt(a), a > 0 in twice the range (a quotient of two values in range).
@@ -93,7 +114,14 @@ __device__ __forceinline__ double sqrt64(double a, const Fma64 &X) {
     const double g0 = X.mul(a, y);
     const double d = fma(-g0, h0, 0.5);
     const double g = fma(g0, d, g0), h = fma(h0, d, h0);
-    return fma(fma(-g, g, a), h, g);
+    const double z = fma(fma(-g, g, a), h, g);
+    // With a = A 2^(e - 52) and z = Z 2^(half - 52), z is the rounded root if and only if
+    // -Z < A 2^(52 + odd) - Z^2 <= Z; the difference is small, so its low 64 bits are all of it.
+    // (z = 2^half, rounded up from a mantissa of ones, is one too high by the same comparison.)
+    const long long zb = __double_as_longlong(z);
+    const unsigned long long Z = ((unsigned long long)zb & 0xfffffffffffffull) | 0x10000000000000ull;
+    const long long R = (long long)(((unsigned long long)((unsigned)lo << (20 + odd)) << 32) - Z * Z);
+    return __longlong_as_double(zb + (R > (long long)Z) - (R <= -(long long)Z));
 }
 
 }  // namespace hydro

@@ -3,9 +3,9 @@
 // on-device dt control block.
 //
 // Two arithmetic modes, chosen by the element type:
-//  * double: every operation is written in the order of the plain formulas (divisions stay
-//    divisions, no reciprocals), and the FP64 translation units are compiled with
-//    --fmad=false, so each operation is one correctly rounded IEEE operation;
+//  * double: the results of the plain formulas, each operation correctly rounded in the formulas'
+//    order.  The FP64 translation units are compiled with --fmad=false; quotients, roots and
+//    comparisons are those of exact64.cuh, which give the IEEE results by fewer FP64 operations;
 //  * float:  the stencil runs in FP32 with fused multiply-adds and the approximate MUFU
 //    reciprocal and square root (rcp.approx / sqrt.approx).
 #pragma once
@@ -342,7 +342,7 @@ __device__ __forceinline__ void hllc(double rl, const double (&vl)[D], double pl
     const double num = X.sub(X.add(X.sub(pr, pl), X.mul(rul, sl)), X.mul(rur, sr));
     const double den = X.sub(ml, mr);
     ok = ok && in_range(den) && (in_range(num) || is_zero(num));
-    const double Ss = X.div(num, den, recip64(den));
+    const double Ss = X.div_by_negative(num, den, recip64(den));
     const bool left = ge0(SL) || ge0(Ss);
     const bool star = !ge0(SL) && (ge0(Ss) || gt0(SR));
     const double r = left ? rl : rr, p = left ? pl : pr, S = left ? SL : SR;
