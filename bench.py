@@ -276,9 +276,9 @@ def run_ours(args):
     del V
     S = hydro.Solver((n, n, n), GAMMA, bc="periodic", dtype=torch.float32, cfl=CFL,
                      variant=dict(staging=args.staging) if args.staging else None)
-    variant = S.variant()
-    variant = {"tile": list(variant["tile"]), "march": variant["march"],
-               "split": "fused dt reduction" if variant["split"] == 2 else "separate CFL pass",
+    variant, launch = S.variant(), S.launch()
+    variant = {"tile": list(variant["tile"]), "kernel": launch["kernel"], "march": launch["march"],
+               "split": "fused dt reduction" if launch["split"] == 2 else "separate CFL pass",
                "staging": {1: "look-ahead", 2: "at use", 3: "TMA"}[variant["staging"]],
                "occupancy": variant["occupancy"]}
     # measured FMA throughput of this GPU (the FP32 roofline's denominator), before the warm-up
@@ -596,7 +596,7 @@ def run_kh2d(args):
     U = hydro.prim_to_cons(V, 5.0 / 3.0).to(dtype).contiguous()
     del V
     S = hydro.Solver((n, n), 5.0 / 3.0, bc="periodic", dtype=dtype, cfl=CFL)
-    variant = S.variant()
+    variant, launch = S.variant(), S.launch()
     S.step(U, args.warmup)
     torch.cuda.synchronize()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -638,8 +638,9 @@ def run_kh2d(args):
             "dtype": "f64" if f64 else "f32", "data": "synthetic",
             "config": {"workload": f"2D periodic {n}^2 shear layer, gamma 5/3, {prec}",
                        "l2": f"state {4 * esz * ncell / 2**20:.0f} MiB vs 129 MB L2; no flush",
-                       "variant": {"tile": list(variant["tile"]), "march": variant["march"],
-                                   "split": variant["split"], "occupancy": variant["occupancy"]}},
+                       "variant": {"tile": list(variant["tile"]), "kernel": launch["kernel"],
+                                   "march": launch["march"], "split": launch["split"],
+                                   "occupancy": variant["occupancy"]}},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "traffic": None, "kernel": dom,
                          "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)"},

@@ -100,11 +100,11 @@ typedef struct {
  *                   (tile, chunk) work items fill the GPU's resident CTAs three times (row
  *                   tiles: twice), the one with the least 0.5 x chunks + 0.3 x planes of the
  *                   last chunk, else 8 (row tiles: 16); FP64: 64 in dim 3, 16 for row tiles).
- *                   Where no march is named, the FP32 strip kernels (below) and the FP64 3D
- *                   tiles choose the planes of a chunk themselves from the grid and the GPU, and
- *                   hydro_get_variant reports the default above.  On the 3D strip kernels a
- *                   named march is an upper bound where its chunks make fewer than three waves
- *                   of CTAs: they take between half of it and all of it, evenly.
+ *                   On the FP32 strip kernels (below) and the FP64 3D tiles the default, named
+ *                   or not, stands for the kernels' own choice from the grid and the GPU, which
+ *                   hydro_get_launch returns.  On the 3D strip kernels any other march is an
+ *                   upper bound where its chunks make fewer than six waves of CTAs: they take
+ *                   between half of it and all of it, evenly.
  *   split:          fusion split.  0 = library default (fused for marching tiles, separate
  *                   for one-plane tiles); 1 = a separate CFL pass after RK stage 2 (one more
  *                   launch and one more read of the state per step); 2 = the CFL signal and
@@ -138,14 +138,13 @@ typedef struct {
  * staging and nothing manifest run kernels whose warps own strips of 64 columns, two cells per
  * lane, and march with everything in registers.  Of a row tile's width they take one warp per 64
  * columns; staging and occupancy do not apply to them.  The FP64 tile 32 x 8 of dim 2 runs strips
- * of 32 columns, one cell per lane, with periodic and outflow boundaries, and unless the variant
- * names a split reduces dt in stage 2 (reported: the tile's default, 1).  Grids of dim 1 of 32 to 2048 cells with
- * periodic or outflow ends run whole chunks of steps in one launch, whatever the variant.
- * Library defaults (measured on GB300): dim 3 FP32 tile 16 x 8 (march from the grid size: 96
- * at 512^3), FP64 32 x 8, march 64; dim 2 FP32 row tile 256 x 1 (march from the grid size: 16
- * at 2048^2, 64 at 4096^2); dim 2 FP64 tile 32 x 8; dim 1 tile 128.  A variant that names a tile other than the default gets that
- * tile's default march (as above in dim 3, 16 for row tiles) and budget unless it names them
- * too.
+ * of 32 columns, one cell per lane, with periodic and outflow boundaries, which reduce dt in stage
+ * 2 whatever the split.  Grids of dim 1 of 32 to 2048 cells with periodic or outflow ends run
+ * whole chunks of steps in one launch, whatever the variant.
+ * Library defaults (measured on GB300): dim 3 FP32 tile 16 x 8, FP64 32 x 8; dim 2 FP32 row tile
+ * 256 x 1, FP64 tile 32 x 8; dim 1 tile 128.  A variant that names a tile other than the default
+ * gets that tile's default march (as above in dim 3, 16 for row tiles) and budget unless it names
+ * them too.
  * Every variant computes the same step; they differ in speed only. */
 typedef struct {
     int32_t tile_x;
@@ -207,9 +206,21 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
                  double cfl, const hydro_variant_t *variant, void *workspace,
                  size_t workspace_bytes, void *stream, hydro_ctx_t **out);
 
-/* The variant a context runs: the one given to hydro_create with every default filled in
- * (split spelled 1 = separate CFL pass, 2 = fused).  Errors: HYDRO_EINVAL (null pointer). */
+/* The variant of a context: the one given to hydro_create with every default filled in (split
+ * spelled 1 = separate CFL pass, 2 = fused).  A context created with it runs the same launches.
+ * Errors: HYDRO_EINVAL (null pointer). */
 int hydro_get_variant(const hydro_ctx_t *ctx, hydro_variant_t *out);
+
+/* What a context's steps launch, where the kernels choose for themselves:
+ *   kernel  HYDRO_KERNEL_TILE (tiles of shared memory, march as in the variant or the FP64 tiles'
+ *           choice), HYDRO_KERNEL_STRIP (strips per warp) or HYDRO_KERNEL_LINE (dim 1, whole runs)
+ *   march   rows (dim 2) or planes (dim 3) that a warp or CTA advances through; 0 for the line
+ *   split   1 = a separate CFL pass after stage 2, 2 = the dt reduction inside the steps' kernels
+ * Errors: HYDRO_EINVAL (null pointer). */
+#define HYDRO_KERNEL_TILE 0
+#define HYDRO_KERNEL_STRIP 1
+#define HYDRO_KERNEL_LINE 2
+int hydro_get_launch(const hydro_ctx_t *ctx, int32_t *kernel, int32_t *march, int32_t *split);
 
 int hydro_destroy(hydro_ctx_t *ctx);
 

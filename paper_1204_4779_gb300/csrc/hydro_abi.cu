@@ -177,8 +177,9 @@ void default_variant(int prec, int dim, hydro_variant_t *v) {
     }
 }
 
-// Reported default march of a 3D FP32 grid (a variant that names no march; the shared-memory tiles
-// run it, the strip kernels take hydro::default_strip_planes): among marches 8, 16, 32, ..., 128
+// Default march of a 3D FP32 grid (a variant that names no march): the shared-memory tiles run it,
+// and naming it leaves the strip kernels their own choice (hydro::default_strip_planes), as naming
+// none does.  Among marches 8, 16, 32, ..., 128
 // whose items fill the GPU's resident CTAs at least three times, the one with the least modelled
 // overhead: 0.5 plane per chunk (the prologue) plus 0.3 times the last chunk's planes (the
 // launch's tail); 8 when none fills them three times.  The weights were fitted to the
@@ -216,8 +217,8 @@ int default_march_3d(const int64_t n[3], const hydro_variant_t &v, int sm_count)
     return choose_march(tiles, n[2], resident_slots(v, sm_count), 3.0, kMarch, 9, 8);
 }
 
-// Planes a CTA of the FP64 3D tiles marches through when the variant names no march (the reported
-// default stays 64): one CTA of 256 threads fits an SM and keeps its FP64 pipe busy, so a launch
+// Planes a CTA of the FP64 3D tiles marches through when the variant names no march, or 64, the
+// default it stands for: one CTA of 256 threads fits an SM and keeps its FP64 pipe busy, so a launch
 // takes (m + 0.7) x (CTAs the busiest SM gets), a chunk's prologue (four recoveries, one face of
 // three) counted as 0.7 planes.  97 x 83 x 75 in chunks of 64 made 88 CTAs for 152 SMs.
 int default_march_f64_3d(const int64_t n[3], const hydro_variant_t &v, int sm_count) {
@@ -236,14 +237,22 @@ int default_march_f64_3d(const int64_t n[3], const hydro_variant_t &v, int sm_co
     return best;
 }
 
-// Reported default march of the 2D FP32 row tiles (a variant that names no march), with the same
-// cost and marches 8, 16, 32, 64, 128 whose items fill the resident CTAs twice; 16 when none does.
-// It is what hydro_get_variant names; a warp of the strip kernels takes
-// hydro::default_strip_rows instead.
+// Default march of the 2D FP32 row tiles (a variant that names no march), with the same cost and
+// marches 8, 16, 32, 64, 128 whose items fill the resident CTAs twice; 16 when none does.  It
+// stands for the strip kernels' own choice, hydro::default_strip_rows, named or not.
 int default_march_rows(const int64_t n[3], const hydro_variant_t &v, int sm_count) {
     static const int kMarch[] = {8, 16, 32, 64, 128};
     const long long strips = (n[0] + v.tile_x - 1) / v.tile_x;
     return choose_march(strips, n[1], resident_slots(v, sm_count), 2.0, kMarch, 5, 16);
+}
+
+// SMs of the current device; 0 where it cannot be asked.
+int device_sms() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return sms;
 }
 
 // The variants the 3D strip kernels run (stage_strip3.cu).
@@ -325,11 +334,11 @@ struct hydro_ctx {
     double lo[3] = {0, 0, 0};
     void *frame[5] = {};
     hydro_variant_t var = {};
-    int strip_rows = 0;      // rows of a warp of the strip kernels of dim 2: FP32 row tiles without
-                             // a named march, the FP64 32 x 8 tile
+    int strip_rows = 0;      // rows of a warp of the strip kernels of dim 2: FP32 row tiles with
+                             // the default march, the FP64 32 x 8 tile
     int split = 0;           // 1: a separate CFL pass after stage 2
-    int march = 1;           // planes of a chunk: the variant's, or where it names none the
-                             // choice of the 3D strip kernels or of the FP64 tiles
+    int march = 1;           // planes of a chunk: the variant's, or the choice of the 3D strip
+                             // kernels or of the FP64 tiles
     Layout lay = {};
     unsigned char *ws = nullptr;
     Ctrl *ctrl = nullptr;
@@ -728,38 +737,27 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
         if (hydro::frame_cells(grid->dim, grid->n[0], grid->dim >= 2 ? grid->n[1] : 1) >= (1LL << 31))
             return HYDRO_EUNSUPPORTED;  // the ring's int indices
     }
-    const bool rows = grid->dim == 2 && var.tile_y == 1;
+    // The march: the variant's, or the default of the grid.  The default stands for the kernels' own
+    // choice, named or not, so that the variant a context reports selects the same launches again.
+    const bool rows = grid->dim == 2 && var.tile_y == 1, strips = strips3(prec, grid->dim, var);
+    const int sms = device_sms();
+    const int64_t extent = grid->n[grid->dim - 1];
+    int standard = grid->dim == 3 ? 64 : 16;
+    if (sms && prec == HYDRO_F32 && grid->dim == 3) standard = default_march_3d(grid->n, var, sms);
+    if (sms && prec == HYDRO_F32 && rows) standard = default_march_rows(grid->n, var, sms);
+    if ((grid->dim == 3 || rows) && !(variant && variant->march)) var.march = standard;
+    const bool own = sms && (var.march < extent ? var.march : extent) == (standard < extent ? standard : extent);
     int strip_rows = 0, own_march = 0;
-    if (grid->dim == 2 && prec == HYDRO_F64 && var.tile_x == 32 && var.tile_y == 8 &&
-        !(ana_axes | ex_axes)) {
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-            strip_rows = hydro::default_row64_rows(grid->n[0], grid->n[1], sms);
-    }
-    if (grid->dim == 3 && prec == HYDRO_F64 && !(variant && variant->march)) {
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-            own_march = default_march_f64_3d(grid->n, var, sms);
-    }
-    if ((grid->dim == 3 || rows) && prec == HYDRO_F32 && !(variant && variant->march)) {
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-            var.march = rows ? default_march_rows(grid->n, var, sms)
-                             : default_march_3d(grid->n, var, sms);
-        if (rows)
-            strip_rows = hydro::default_strip_rows(grid->n[0], grid->n[1], sms);
-        else if (strips3(prec, grid->dim, var))
-            own_march = hydro::default_strip_planes(grid->n[0], grid->n[1], grid->n[2], sms);
-    }
-    if (strips3(prec, grid->dim, var) && variant && variant->march) {
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-            own_march = hydro::fitted_strip_planes(grid->n[0], grid->n[1], grid->n[2], var.march, sms);
-    }
+    if (rows && prec == HYDRO_F32 && own)
+        strip_rows = hydro::default_strip_rows(grid->n[0], grid->n[1], sms);
+    if (sms && grid->dim == 2 && prec == HYDRO_F64 && var.tile_x == 32 && var.tile_y == 8 &&
+        !(ana_axes | ex_axes))
+        strip_rows = hydro::default_row64_rows(grid->n[0], grid->n[1], sms);
+    if (grid->dim == 3 && prec == HYDRO_F64 && own)
+        own_march = default_march_f64_3d(grid->n, var, sms);
+    if (sms && strips)
+        own_march = own ? hydro::default_strip_planes(grid->n[0], grid->n[1], grid->n[2], sms)
+                        : hydro::fitted_strip_planes(grid->n[0], grid->n[1], grid->n[2], var.march, sms);
     const Layout lay = layout_for(grid->dim, grid->n, ncell, prec, var.manifest);
     if (workspace_bytes < lay.total) return HYDRO_EINVAL;
     // grid-dimension limits of the stage launch
@@ -793,9 +791,9 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
     c->cfl = cfl;
     c->var = var;
     c->strip_rows = strip_rows;
-    // the FP64 strips keep the new states in registers: the dt reduction joins stage 2 unless the
-    // variant names the separate pass (the reported default belongs to the tile kernels)
-    c->split = strip_rows && prec == HYDRO_F64 && !(variant && variant->split) ? 0 : var.split;
+    // the FP64 strips keep the new states in registers: the dt reduction joins stage 2 (the tile's
+    // default, a separate pass, stands for that too)
+    c->split = strip_rows && prec == HYDRO_F64 ? 0 : var.split;
     c->march = own_march ? own_march : var.march;
     if (marching && c->march > c->n[c->dim - 1]) c->march = c->n[c->dim - 1];
     c->lay = lay;
@@ -852,6 +850,17 @@ int hydro_get_variant(const hydro_ctx_t *c, hydro_variant_t *out) {
     if (!c || !out) return HYDRO_EINVAL;
     *out = c->var;
     out->split = c->var.split ? 1 : 2;  // the ABI's spelling: 1 separate CFL pass, 2 fused
+    return HYDRO_OK;
+}
+
+int hydro_get_launch(const hydro_ctx_t *c, int32_t *kernel, int32_t *march, int32_t *split) {
+    if (!c || !kernel || !march || !split) return HYDRO_EINVAL;
+    const bool line = c->line_ctas != 0;
+    const bool strips = c->strip_rows || (c->prec == HYDRO_F32 && c->dim == 2 && c->var.tile_y == 1) ||
+                        strips3(c->prec, c->dim, c->var);
+    *kernel = line ? HYDRO_KERNEL_LINE : (strips ? HYDRO_KERNEL_STRIP : HYDRO_KERNEL_TILE);
+    *march = line ? 0 : (c->strip_rows ? c->strip_rows : c->march);
+    *split = line || !c->split ? 2 : 1;
     return HYDRO_OK;
 }
 

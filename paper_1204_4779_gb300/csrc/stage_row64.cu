@@ -16,8 +16,7 @@ cudaError_t stage_row64(const StageLaunch &L, cudaStream_t st) {
     if (items < 1 || items >= (1LL << 31) - 4) return cudaErrorInvalidValue;
     A.items = (int)items;
     constexpr int warps = kRow64Threads / 32;
-    const auto k = L.stage == 1 ? row64_stage_kernel<1, false>
-                                : (L.split ? row64_stage_kernel<2, false> : row64_stage_kernel<2, true>);
+    const auto k = L.stage == 1 ? row64_stage_kernel<1, false> : row64_stage_kernel<2, true>;
     k<<<(unsigned)((items + warps - 1) / warps), kRow64Threads, 0, st>>>(A);
     return cudaGetLastError();
 }

@@ -29,6 +29,7 @@ HYDRO_F64, HYDRO_F32 = 0, 1
 EXPORTS = (
     "hydro_version", "hydro_strerror", "hydro_last_cuda_error", "hydro_variant_supported",
     "hydro_workspace_bytes", "hydro_workspace_bytes_variant", "hydro_create", "hydro_get_variant",
+    "hydro_get_launch",
     "hydro_destroy", "hydro_set_stream",
     "hydro_step",
     "hydro_step_host", "hydro_step_host_async", "hydro_set_scheme", "hydro_set_analytic", "hydro_analytic_state", "hydro_cfl_dt", "hydro_totals", "hydro_status", "hydro_prim_to_cons",
@@ -97,6 +98,7 @@ def load_library(path: str = LIB_PATH, build_if_missing: bool = True):
                               P(vp)], ctypes.c_int),
             "hydro_destroy": ([vp], ctypes.c_int),
             "hydro_get_variant": ([vp, P(Variant)], ctypes.c_int),
+            "hydro_get_launch": ([vp, P(i32), P(i32), P(i32)], ctypes.c_int),
             "hydro_set_stream": ([vp, vp], ctypes.c_int),
             "hydro_set_scheme": ([vp, i32, i32], ctypes.c_int),
             "hydro_set_analytic": ([vp, i32, dbl, dbl], ctypes.c_int),
@@ -291,11 +293,21 @@ class Solver:
             pass
 
     def variant(self) -> dict:
-        """The variant this context runs, defaults filled in (hydro_get_variant)."""
+        """The variant of this context, defaults filled in; a solver created with it runs the same
+        launches (hydro_get_variant).  Where a default march stands for the kernels' own choice,
+        launch() tells what that is."""
         v = Variant()
         _check(self.lib.hydro_get_variant(self.ctx, ctypes.byref(v)), "hydro_get_variant")
         return {"tile": (v.tile_x, v.tile_y), "march": v.march, "split": v.split,
                 "staging": v.staging, "occupancy": v.occupancy, "manifest": v.manifest}
+
+    def launch(self) -> dict:
+        """What the steps launch (hydro_get_launch): the kernel ("tile", "strip" or "line"), the
+        rows or planes it marches through (0 for the line) and the split that runs."""
+        v = [ctypes.c_int32() for _ in range(3)]
+        _check(self.lib.hydro_get_launch(self.ctx, *[ctypes.byref(x) for x in v]), "hydro_get_launch")
+        return {"kernel": ("tile", "strip", "line")[v[0].value], "march": v[1].value,
+                "split": v[2].value}
 
     # -- helpers ---------------------------------------------------------------------------
     def empty_state(self) -> torch.Tensor:

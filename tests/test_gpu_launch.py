@@ -1,0 +1,62 @@
+"""What a context launches (hydro_get_launch), and that the variant it reports selects the same
+launches when it is passed back, whichever kernels chose their march for themselves."""
+import pytest
+
+from paper_1204_4779_gb300 import hydro
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+F32, F64 = torch.float32, torch.float64
+
+GRIDS = [((1024,), F64), ((2500,), F32), ((300, 77), F64), ((1024, 1024), F64), ((3001, 2003), F32),
+         ((512, 512), F32), ((40, 36, 5), F32), ((128, 128, 128), F32), ((256, 256, 256), F32),
+         ((97, 83, 75), F64), ((40, 36, 100), F64)]
+
+
+@pytest.mark.parametrize("shape,dtype", GRIDS)
+@pytest.mark.parametrize("bc", ["periodic", "outflow"])
+def test_a_reported_variant_runs_the_same_launches(shape, dtype, bc):
+    variants = [None]
+    if len(shape) == 3:
+        variants += [dict(march=20), dict(march=64), dict(split=1)]
+        if dtype == F32:
+            variants += [dict(staging=2), dict(staging=3), dict(tile=(32, 8)), dict(manifest=2)]
+    elif len(shape) == 2:
+        variants += [dict(split=1), dict(split=2)]
+        variants += [dict(march=16), dict(march=64), dict(tile=(64, 1))] if dtype == F32 else \
+            [dict(tile=(128, 1)), dict(tile=(128, 1), march=7)]
+    for var in variants:
+        A = hydro.Solver(shape, 1.4, bc=bc, dtype=dtype, variant=var)
+        B = hydro.Solver(shape, 1.4, bc=bc, dtype=dtype, variant=A.variant())
+        assert A.variant() == B.variant() and A.launch() == B.launch(), (var, A.launch(), B.launch())
+        A.close()
+        B.close()
+
+
+@pytest.mark.parametrize("shape,dtype,variant,want", [
+    ((1024,), F64, None, ("line", 0, 2)), ((1024,), F32, None, ("line", 0, 2)),
+    ((2049,), F64, None, ("tile", 1, 1)),
+    ((512, 512), F32, None, ("strip", 2, 2)), ((1024, 1024), F32, None, ("strip", 8, 2)),
+    ((2048, 2048), F32, None, ("strip", 32, 2)), ((3001, 2003), F32, None, ("strip", 48, 2)),
+    ((4096, 4096), F32, None, ("strip", 24, 2)),
+    ((1024, 1024), F32, dict(march=12, split=1), ("strip", 12, 1)),
+    ((1024, 1024), F64, None, ("strip", 21, 2)), ((300, 77), F64, dict(tile=(128, 1)), ("tile", 16, 2)),
+    ((128, 128, 128), F32, None, ("strip", 22, 2)), ((256, 256, 256), F32, None, ("strip", 26, 2)),
+    ((512, 512, 512), F32, None, ("strip", 128, 2)), ((512, 512, 512), F32, dict(march=40), ("strip", 40, 2)),
+    ((128, 128, 128), F32, dict(march=40, staging=3), ("tile", 40, 2)),
+    ((97, 83, 75), F64, None, ("tile", 25, 2)), ((97, 83, 75), F64, dict(march=32, split=1), ("tile", 32, 1))])
+def test_launches_that_run(shape, dtype, variant, want):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the expected marches are those of a 152-SM GPU")
+    S = hydro.Solver(shape, 1.4, dtype=dtype, variant=variant)
+    got = S.launch()
+    S.close()
+    assert (got["kernel"], got["march"], got["split"]) == want
+
+
+def test_null_arguments():
+    import ctypes
+    lib = hydro.load_library()
+    v = ctypes.c_int32()
+    assert lib.hydro_get_launch(None, ctypes.byref(v), ctypes.byref(v), ctypes.byref(v)) == hydro.HYDRO_EINVAL
