@@ -137,7 +137,8 @@ typedef struct {
  * Strip kernels: the FP32 row tiles of dim 2 and, in dim 3, the FP32 tile 16 x 8 with look-ahead
  * staging and nothing manifest run kernels whose warps own strips of 64 columns, two cells per
  * lane, and march with everything in registers.  Of a row tile's width they take one warp per 64
- * columns; staging and occupancy do not apply to them.  The FP64 tile 32 x 8 of dim 2 runs strips
+ * columns; staging and occupancy do not apply to them.  (Grids of dim 3 too narrow for the strips
+ * run the 16 x 8 tiles, each plane loaded when it is staged.)  The FP64 tile 32 x 8 of dim 2 runs strips
  * of 32 columns, one cell per lane, with periodic and outflow boundaries, which reduce dt in stage
  * 2 whatever the split.  Grids of dim 1 of 32 to 2048 cells with periodic or outflow ends run
  * whole chunks of steps in one launch, whatever the variant.

@@ -336,6 +336,7 @@ struct hydro_ctx {
     hydro_variant_t var = {};
     int strip_rows = 0;      // rows of a warp of the strip kernels of dim 2: FP32 row tiles with
                              // the default march, the FP64 32 x 8 tile
+    bool narrow = false;     // dim 3: a narrow grid, on the 16 x 8 tiles instead of the strips
     int split = 0;           // 1: a separate CFL pass after stage 2
     int march = 1;           // planes of a chunk: the variant's, or the choice of the 3D strip
                              // kernels or of the FP64 tiles
@@ -387,7 +388,7 @@ hydro::StageLaunch stage_args(const hydro_ctx *c, const hydro_state_t *s, int st
     L.rows = c->strip_rows;
     L.tile_x = c->var.tile_x;
     L.tile_y = c->var.tile_y;
-    L.prefetch = c->var.staging == 2 ? 0 : (c->var.staging == 3 ? 2 : 1);
+    L.prefetch = c->var.staging == 2 || c->narrow ? 0 : (c->var.staging == 3 ? 2 : 1);
     L.split = c->split;
     L.occupancy = c->var.occupancy;
     L.manifest = c->var.manifest == 2 ? 1 : (c->var.manifest == 3 ? 2 : 0);
@@ -758,6 +759,9 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
     if (sms && strips)
         own_march = own ? hydro::default_strip_planes(grid->n[0], grid->n[1], grid->n[2], sms)
                         : hydro::fitted_strip_planes(grid->n[0], grid->n[1], grid->n[2], var.march, sms);
+    const bool narrow = sms && strips && hydro::strip3_narrow(grid->n[0], grid->n[1], grid->n[2],
+                                                              own_march, var.march, sms);
+    if (narrow) own_march = 0;  // the tiles run the variant's march
     const Layout lay = layout_for(grid->dim, grid->n, ncell, prec, var.manifest);
     if (workspace_bytes < lay.total) return HYDRO_EINVAL;
     // grid-dimension limits of the stage launch
@@ -795,6 +799,7 @@ int hydro_create(const hydro_grid_t *grid, double gamma, const int32_t bc[3], in
     // default, a separate pass, stands for that too)
     c->split = strip_rows && prec == HYDRO_F64 ? 0 : var.split;
     c->march = own_march ? own_march : var.march;
+    c->narrow = narrow;
     if (marching && c->march > c->n[c->dim - 1]) c->march = c->n[c->dim - 1];
     c->lay = lay;
     c->ws = static_cast<unsigned char *>(workspace);
@@ -857,7 +862,7 @@ int hydro_get_launch(const hydro_ctx_t *c, int32_t *kernel, int32_t *march, int3
     if (!c || !kernel || !march || !split) return HYDRO_EINVAL;
     const bool line = c->line_ctas != 0;
     const bool strips = c->strip_rows || (c->prec == HYDRO_F32 && c->dim == 2 && c->var.tile_y == 1) ||
-                        strips3(c->prec, c->dim, c->var);
+                        (strips3(c->prec, c->dim, c->var) && !c->narrow);
     *kernel = line ? HYDRO_KERNEL_LINE : (strips ? HYDRO_KERNEL_STRIP : HYDRO_KERNEL_TILE);
     *march = line ? 0 : (c->strip_rows ? c->strip_rows : c->march);
     *split = line || !c->split ? 2 : 1;

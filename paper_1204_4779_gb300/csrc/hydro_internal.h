@@ -79,6 +79,8 @@ cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare
 int default_strip_planes(long long nx, long long ny, long long nz, int sm_count);
 // and for a named march of m planes (at most m)
 int fitted_strip_planes(long long nx, long long ny, long long nz, int m, int sm_count);
+// narrow grids that the 16 x 8 tile kernel steps faster than the strips
+bool strip3_narrow(long long nx, long long ny, long long nz, int m_strips, int m_tiles, int sm_count);
 int default_strip_rows(long long nx, long long ny, int sm_count);
 
 // Whole runs of small 1D grids (line_kernel.cuh): up to n_steps steps from the control block's dt

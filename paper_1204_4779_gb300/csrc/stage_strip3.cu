@@ -127,4 +127,24 @@ int fitted_strip_planes(long long nx, long long ny, long long nz, int m, int sm_
     return best;
 }
 
+// Whether the 16 x 8 tile kernel (no look-ahead, m_tiles planes a CTA) is the faster one of a grid
+// whose strips would march m_strips planes: grids so narrow that less than two thirds of a strip
+// CTA's 448 lanes own a cell, and large enough to fill the GPU with tiles.  A tile launch of
+// w waves (six CTAs an SM) takes (m + 1) x w, or (0.4 + 0.6 w) where w < 1, in units of 1.2 planes
+// of the strips' strip3_cost; both models fitted to 113 grids, the choice at worst 7 % from the
+// better one.  Measured on GB300, us per step, tiles of the earlier version / strips / tiles now:
+//   29x200x200    88.0  101.5   80.5*     61x200x200   147   156   140*
+//   32x200x200    87.4   92.7   78.8*     64x200x200   148   143*  143
+//   33x200x200   116    100.8* 109.8      16x200x200   57.7  54.4  49.7*
+//   4x384x384    133    204    120*       16x64x48     34.0  17.6* 31.8
+bool strip3_narrow(long long nx, long long ny, long long nz, int m_strips, int m_tiles, int sm_count) {
+    if ((double)nx * (double)ny >= 0.66 * 448.0 * strip3_tiles(nx, ny)) return false;
+    const long long ctas = ((nx + 15) / 16) * ((ny + 7) / 8) * ((nz + m_tiles - 1) / m_tiles);
+    const double waves = (double)ctas / (6.0 * (sm_count > 0 ? sm_count : 1));
+    if (waves < 0.3) return false;
+    const double planes = (double)(m_tiles < nz ? m_tiles : nz) + 1.0;
+    return 1.2 * planes * (waves < 1.0 ? 0.4 + 0.6 * waves : waves) <
+           strip3_cost(nx, ny, nz, m_strips, sm_count);
+}
+
 }  // namespace hydro

@@ -2,7 +2,7 @@
 launches when it is passed back, whichever kernels chose their march for themselves."""
 import pytest
 
-from paper_1204_4779_gb300 import hydro
+from paper_1204_4779_gb300 import hydro, inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -53,6 +53,30 @@ def test_launches_that_run(shape, dtype, variant, want):
     got = S.launch()
     S.close()
     assert (got["kernel"], got["march"], got["split"]) == want
+
+
+def _state(shape):
+    V = torch.from_numpy(inputs.smooth(shape, seed=5, vmax=0.3)).cuda()
+    return hydro.prim_to_cons(V, 1.4).to(F32).contiguous()
+
+
+@pytest.mark.parametrize("shape,kernel", [
+    ((29, 200, 200), "tile"), ((32, 150, 150), "tile"), ((4, 384, 384), "tile"), ((61, 300, 100), "tile"),
+    ((64, 16, 384), "tile"), ((28, 200, 200), "strip"), ((60, 150, 150), "strip"), ((29, 64, 48), "strip"),
+    ((33, 200, 200), "strip"), ((2, 3, 5), "strip"), ((128, 128, 128), "strip")])
+def test_narrow_grids_run_the_faster_kernel_with_the_same_result(shape, kernel):
+    """One chunk of all planes leaves too few tiles for the rule, so that form runs the strips: the
+    states agree bit for bit."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the rule's lines are those of a 152-SM GPU")
+    A = hydro.Solver(shape, 1.4, bc=["periodic", "outflow", "periodic"], dtype=F32)
+    B = hydro.Solver(shape, 1.4, bc=["periodic", "outflow", "periodic"], dtype=F32,
+                     variant=dict(march=max(shape[2], 9)))
+    assert A.launch()["kernel"] == kernel and B.launch()["kernel"] == "strip"
+    U = _state(shape)
+    W = U.clone()
+    assert A.step(U, 5) == B.step(W, 5)
+    assert torch.equal(U, W)
 
 
 def test_null_arguments():
