@@ -2,7 +2,7 @@
 launches when it is passed back, whichever kernels chose their march for themselves."""
 import pytest
 
-from paper_1204_4779_gb300 import hydro, inputs
+from paper_1204_4779_gb300 import hydro, inputs, tuner
 
 pytestmark = pytest.mark.gpu
 
@@ -77,6 +77,24 @@ def test_narrow_grids_run_the_faster_kernel_with_the_same_result(shape, kernel):
     W = U.clone()
     assert A.step(U, 5) == B.step(W, 5)
     assert torch.equal(U, W)
+
+
+@pytest.mark.parametrize("shape", [(512, 512), (1024, 1024), (2048, 2048), (4096, 4096), (300, 77),
+                                   (64, 64, 64), (128, 128, 128), (160, 160, 160), (40, 36, 30)])
+def test_the_tuner_can_name_the_default(shape):
+    """Some variant of the tuner's space runs the launches of a solver created without one, so the
+    best one found is no slower than that."""
+    S = hydro.Solver(shape, 1.4, dtype=F32)
+    want, default = S.launch(), S.variant()
+    S.close()
+    space = tuner.Space(len(shape))
+    named = [v for v in map(space.variant, space.all_genomes())
+             if all(default[k] == x for k, x in v.items())]
+    assert len(named) == 1
+    S = hydro.Solver(shape, 1.4, dtype=F32, variant=named[0])
+    got = S.launch()
+    S.close()
+    assert got == want
 
 
 def test_null_arguments():
