@@ -693,8 +693,8 @@ def run_batched(args):
             "config": {"workload": "4096 independent 2D grids, sides log-uniform on [32, 512] "
                                    "(seed 1204477904), smooth seeded data, FP32",
                        "cells": ncell, "l2": "inputs larger than L2 (1.9 GB state); no flush",
-                       "variant": "library default: row tiles of 32 columns marching 32 rows "
-                                  "along y, one work item per strip and chunk"},
+                       "variant": "library default: strips of 60 columns marching along y, one "
+                                  "work item per strip and chunk of rows"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm,
                          "traffic": _ncu_record("per_launch_bytes", dom, "ncu_counters_batched.json",

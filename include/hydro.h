@@ -128,8 +128,7 @@ typedef struct {
  *                   stores the primitive planes of the stage's input, which the stage kernel
  *                   reads instead of U; 3 = F: the stage kernel stores every face flux and a
  *                   pass applies AddFlux (and stage 2's dt reduction).  All three compute the
- *                   same step: bit for bit in FP64; in FP32 to rounding (where V or a flux
- *                   stays in registers the compiler may fuse a product into its consumer).
+ *                   same step: bit for bit in FP64, in FP32 to rounding.
  *                   dim 3 only, for the tiles compiled with them (FP32
  *                   16 x 8, 32 x 8, 16 x 16; FP64 32 x 8), with look-ahead staging and the
  *                   precision's default budget; 2 and 3 need more workspace
@@ -138,10 +137,10 @@ typedef struct {
  * staging and nothing manifest run kernels whose warps own strips of 64 columns, two cells per
  * lane, and march with everything in registers.  Of a row tile's width they take one warp per 64
  * columns; staging and occupancy do not apply to them.  (Grids of dim 3 too narrow for the strips
- * run the 16 x 8 tiles, each plane loaded when it is staged.)  The FP64 tile 32 x 8 of dim 2 runs strips
- * of 32 columns, one cell per lane, with periodic and outflow boundaries, which reduce dt in stage
- * 2 whatever the split.  Grids of dim 1 of 32 to 2048 cells with periodic or outflow ends run
- * whole chunks of steps in one launch, whatever the variant.
+ * run the 16 x 8 tiles, each plane loaded when it is staged.)  The FP64 tile 32 x 8 of dim 2 runs
+ * strips of 32 columns, one cell per lane, with periodic and outflow boundaries, which reduce dt
+ * in stage 2 whatever the split.  Grids of dim 1 of 32 to 2048 cells with periodic or outflow
+ * ends run whole chunks of steps in one launch, whatever the variant.
  * Library defaults (measured on GB300): dim 3 FP32 tile 16 x 8, FP64 32 x 8; dim 2 FP32 row tile
  * 256 x 1, FP64 tile 32 x 8; dim 1 tile 128.  A variant that names a tile other than the default
  * gets that tile's default march (as above in dim 3, 16 for row tiles) and budget unless it names
@@ -269,10 +268,11 @@ int hydro_set_scheme(hydro_ctx_t *ctx, int32_t order, int32_t riemann);
  * dt is computed on the device from the state at the start of each step (the first from
  * `state` by a CFL pass, later ones in the epilogue of the previous step) and never leaves
  * the device inside the call.  The steps run as CUDA graphs of captured launches (chunks of up
- * to 64 steps; grids of dim 1 of 32 to 2048 cells: up to 2048 steps in one launch); once no further step is to be taken (t_end reached or a failed step) the steps
- * left return at once on the device, and a synchronous call stops launching chunks after
- * that (it reads dt back after each chunk, one chunk late, so n_steps may be a generous
- * bound when t_end is what ends the run).
+ * to 64 steps; grids of dim 1 of 32 to 2048 cells: up to 2048 steps in one launch); once no
+ * further step is to be taken (t_end reached or a failed step) the steps left return at once on
+ * the device, and a synchronous call stops launching chunks after that (it reads dt back after
+ * each chunk, one chunk late, so n_steps may be a generous bound when t_end is what ends the
+ * run).
  * If both t_inout and steps_done are NULL the call is asynchronous and a device-side error
  * is reported by the next synchronising call; otherwise it synchronises and returns
  * HYDRO_ENONFINITE if a step failed. */

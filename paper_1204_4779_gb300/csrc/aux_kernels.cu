@@ -141,8 +141,9 @@ __global__ void __launch_bounds__(kAuxThreads)
         for (int k = 0; k < NV; ++k) acc[k] = {0.0f, 0.0f};
         // four cells a thread and access (chunks then start on multiples of four cells)
         const long long q0 = b0 / 4, q1 = A.wide ? b1 / 4 : q0;
-        // (two groups of four cells in flight; four values are summed exactly in a tree of TwoSums
-        // before they join the running sum: 31 operations instead of 44)
+        // (two groups of four cells in flight; four values are summed in a tree of TwoSums, their
+        // low parts added in FP32, to 2^-48 of the largest, before they join the running sum, which
+        // keeps as much: 31 operations instead of 44)
         auto add4 = [&](int k, const T (&u)[Wide<T>::n]) {
             const DF p = two_sum((float)u[0], (float)u[1]), r = two_sum((float)u[2], (float)u[3]);
             const DF h = two_sum(p.hi, r.hi);

@@ -1,4 +1,4 @@
-// FP32 batched RK-stage kernels (compiled with FMA contraction).
+// FP32 batched RK-stage kernels (FMAs are written out; the compiler contracts none).
 #include "batch_kernel.cuh"
 
 namespace hydro {

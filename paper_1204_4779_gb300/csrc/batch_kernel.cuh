@@ -237,8 +237,8 @@ __global__ void __launch_bounds__(BX, (MinBlocks<T, BX, OCC>::value))
 // FP32 row tiles: an item is a strip of kStripCells columns of one grid and a chunk of `rows`
 // rows, advanced by one warp (row_kernel.cuh), which claims its items by itself.  4096 grids of
 // 32-512 cells a side (121 M cells): 4.46 ms per step with the shared-memory row tiles of 32
-// columns, 2.61 ms so (46 G cell-updates/s; bound by instruction issue).  CTAs of four warps
-// against one: 2.61 / 2.86 ms.
+// columns, 2.78 ms so (44 G cell-updates/s; bound by instruction issue).  CTAs of four warps
+// against one, on another draw of 118 M cells: 2.61 / 2.86 ms.
 template <int STAGE>
 __global__ void __launch_bounds__(kRowThreads, 4) batch_strip_kernel(const BatchArgs<float> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];

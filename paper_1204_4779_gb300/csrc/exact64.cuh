@@ -92,7 +92,8 @@ __device__ __forceinline__ double recip64(double b) {
     const long long z = __double_as_longlong(fma(y, fma(d, d, d), y));
     // B Y = 2^104 or 2^105 minus the remainder, whose low 64 bits are all of it; Y is the rounded
     // reciprocal if and only if |remainder| <= B / 2
-    const unsigned long long B = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)lo;
+    const unsigned long long B =
+        ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)lo;
     const unsigned long long Y = ((unsigned long long)z & 0xfffffffffffffull) | 0x10000000000000ull;
     const long long R = (long long)(0ull - 2ull * (B * Y));
     return __longlong_as_double(z + (R > (long long)B) - (R < -(long long)B));

@@ -292,7 +292,7 @@ __device__ __forceinline__ void chunk_wgrad(const float *z, const float *in, int
 // results equal theirs bit for bit (training amplifies a last bit by orders of magnitude over 200
 // epochs).  The errors y - t go to err, the chunk's sums (the parameters' layout) to
 // part[chunk P].  Training (stepc non-null): CTA 0 advances the Adam step counter, which the update
-// kernel after it reads.  Bound by shared-memory accesses (LSU wavefronts 48 % busy) along a
+// kernel after it reads.  Bound by shared-memory accesses (the LSU's wavefronts 60 % of its peak) along a
 // chain of five dependent passes; 17.6 us of the epoch under a profiler with cold caches.
 __global__ void __cluster_dims__(kTiles, 1, 1) __launch_bounds__(kChunkThreads)
     mlp_chunk_kernel(const float *p, int d, int H, const float *X, const float *t, long long n,

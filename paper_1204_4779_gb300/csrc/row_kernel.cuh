@@ -5,8 +5,9 @@
 // y-neighbours' from the lane's own register pipeline, so nothing waits on another warp, each
 // slope is computed once, and most of the arithmetic serves two cells per instruction.  The rows
 // ahead come by asynchronous copies into a ring in shared memory (a load into registers ahead of
-// its use does not stay ahead: under the register budget it is scheduled back to its use).  The outer two columns on each side are the strip's halo: 60 of 64 columns are
-// stored (the warp repeats its neighbours' work on four columns instead of exchanging them).
+// its use does not stay ahead: under the register budget it is scheduled back to its use).  The
+// outer two columns on each side are the strip's halo: 60 of 64 columns are stored (the warp
+// repeats its neighbours' work on four columns instead of exchanging them).
 //
 // The step is bound by instruction issue, not by HBM or the FP32 pipe: the shared-memory row
 // tiles this replaced executed 380-408 instructions per cell and stage (one cell per thread,

@@ -1,5 +1,5 @@
-// FP32 RK-stage kernels, dims 1 and 2 (compiled with FMA contraction): one-plane tiles, and in
-// dim 2 row tiles that march along y (stage_rows.cu).
+// FP32 RK-stage kernels, dims 1 and 2 (FMAs are written out; the compiler contracts none):
+// one-plane tiles, and in dim 2 row tiles that march along y (stage_rows.cu).
 #include "stage_launch.cuh"
 
 namespace hydro {

@@ -1,5 +1,6 @@
-// FP32 RK-stage kernels, dim 3 (compiled with FMA contraction), both staging depths and both
-// occupancy targets: tiles 32x8, 32x4, 64x4 (the others are in stage_f32_d3b.cu).
+// FP32 RK-stage kernels, dim 3 (FMAs are written out; the compiler contracts none), both
+// staging depths and both occupancy targets: tiles 32x8, 32x4, 64x4 (the others are in
+// stage_f32_d3b.cu).
 #include "stage_launch.cuh"
 
 namespace hydro {

@@ -35,15 +35,16 @@ int row_warps(long long strips, int most) {
     return best;
 }
 
-// Rows a warp marches through when the variant names no march: the least (m + 2) x (waves of the
-// resident warps, plus half a wave of tail once there is more than one).  A chunk's prologue (four
-// rows recovered, one extra face, the first copies' latency) costs about two rows.  Measured on
-// GB300, us per step, shear layer, m = 2 / 4 / 8 / 12 / 16 / 24 / 32 / 64, chosen marked:
-//   512^2     17.2* 18.5  20.6  21.6  23.3  31.7  38.4  66.3
-//   1024^2    42.4  34.2  33.8* 32.8  39.1  40.8  50.4  65.7
-//   2048^2    187   132   107   101   101   98.1  98.7* 103
-//   3001x2003 220   159   143   137   133*  138   138   137
-//   4096^2    551   372   316   303   298   295*  299   305
+// Rows a warp marches through by default: the least (m + 2) x (waves of the resident warps, plus
+// half a wave of tail once there is more than one).  A chunk's prologue (four rows recovered, one
+// extra face, the first copies' latency) costs about two rows.  Measured on GB300, us per step,
+// shear layer, m = 2 / 4 / 8 / 12 / 16 / 24 / 32 / 48 / 64, the rule's choice marked; it is within
+// 2.5 % of the best of each row:
+//   512^2     16.9* 17.9  20.2  21.1  24.8  31.3  38.1  52.1  66.2
+//   1024^2    42.1  34.0  33.6* 32.8  38.8  40.6  50.3  53.0  66.7
+//   2048^2    185   130   106   100   101   97.5  98.2* 107   104
+//   3001x2003 217   158   142   137   133   137   138   136*  136
+//   4096^2    545   369   312   300   295   292*  297   291   302
 int row_march(long long strips, long long ny, int warp_slots) {
     static const int kRows[] = {2, 4, 6, 8, 12, 16, 24, 32, 48, 64};
     int best = 0;

@@ -87,15 +87,15 @@ cudaError_t stage_strip3_f32(const StageLaunch &L, cudaStream_t st, bool prepare
                                             : launch_strip3<32>(L, A, st);
 }
 
-// Planes a CTA marches through when the variant names no march: the least (m + 1.5) x waves, a
-// chunk's prologue counted as 1.5 planes, the last wave of the resident CTAs (two per SM) whole,
-// or 0.62 where no SM gets a second CTA of it.  Measured on GB300, blast, us per step at m = 4 / 8 / 12 / 16 / 24 / 32 / 64 / 96,
-// chosen marked:
-//   64^3   30.0* 31.3  40.7  49.9  68.5  86.8  161
-//   128^3  119   116   112   114   110*  142   164   241
-//   192^3  327   299   296   286   308   279   276*  402
-//   256^3  792   710   686   680   676   664*  664   707
-//   512^3  5651  5025  4822  4719  4610  4582  4560* 4472
+// Planes a CTA marches through by default: the least (m + 1.5) x waves, a chunk's prologue counted
+// as 1.5 planes, the last wave of the resident CTAs (two per SM) whole, or 0.62 where no SM gets a
+// second CTA of it.  Measured on GB300, blast, us per step at m planes, the rule's choice marked;
+// it is within 3 % of the best of each row:
+//   64^3    1: 35.9  2: 31.0  4: 28.6*  6: 31.5  8: 30.3  16: 48.7
+//   128^3   8: 114  12: 110  16: 112  22: 100*  24: 108  32: 139
+//   192^3  16: 279  24: 303  32: 274  48: 310  64: 271*  96: 396
+//   256^3  16: 669  24: 665  26: 671*  32: 653  52: 711  64: 654  86: 689
+//   512^3  32: 4520  64: 4498  74: 4441  86: 4497  96: 4411  128: 4500*  171: 4644
 int default_strip_planes(long long nx, long long ny, long long nz, int sm_count) {
     static const int kPlanes[] = {2, 4, 6, 8, 12, 16, 20, 24, 32, 40, 48, 64, 80, 96, 128};
     int best = 0;

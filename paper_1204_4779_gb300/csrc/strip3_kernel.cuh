@@ -2,12 +2,13 @@
 //
 // A warp owns 64 columns of one row, two neighbouring ones per lane in packed f32x2 pairs (60 are
 // stored, as in row_kernel.cuh; or 32 columns of two rows, 28 stored), and marches through a chunk
-// of z-planes; a CTA is seven such warps one above the other and a helper warp.  The x-neighbours' values come by warp shuffles,
-// the z-neighbours' from the lane's own pipeline, the y-neighbours' through shared memory: each
-// row's V, then the upper face states, then the fluxes of the rows' lower faces, two barriers a
-// plane.  Every slope and every face is computed once.  The helper warp does what belongs to the
-// rows outside the CTA's (V of the two rows on each side, their face states, the face above the
-// last row), so that the rows' warps run the same straight code and none is late at a barrier.
+// of z-planes; a CTA is seven such warps one above the other and a helper warp.  The
+// x-neighbours' values come by warp shuffles, the z-neighbours' from the lane's own pipeline, the
+// y-neighbours' through shared memory: each row's V, then the upper face states, then the fluxes
+// of the rows' lower faces, two barriers a plane.  Every slope and every face is computed once.
+// The helper warp does what belongs to the rows outside the CTA's (V of the two rows on each
+// side, their face states, the face above the last row), so that the rows' warps run the same
+// straight code and none is late at a barrier.
 // Rows of U ahead (own and base) come by cp.async.
 #pragma once
 

@@ -31,7 +31,8 @@
 // arithmetic (GB300's FP64 pipe runs at 1/62 of the FP32 rate).  Each cell recomputes f1 at
 // i-1, i, i+1 from f and g (one FP32 operation each, the neighbours' loads hitting cache), so
 // the tile loop has no barrier; where n is a multiple of four and the arrays are 16-byte
-// aligned a thread takes four consecutive cells with 128-bit loads and stores.  With D = f1[i+1] - f1[i-1] and G = g[i] + g1[i], the energy is
+// aligned a thread takes four consecutive cells with 128-bit loads and stores.  With
+// D = f1[i+1] - f1[i-1] and G = g[i] + g1[i], the energy is
 // K1 sum D^2 + K2 sum G^2, K1 = c^2 dx / (8 dx^2), K2 = dx / 8.  D and G are formed exactly as
 // FP32 pairs (hi + lo) by Knuth's TwoSum, their squares as pairs by the FMA form of Dekker's
 // TwoProduct (dropping lo^2, 2^-48 of the square), and each thread adds them to two running

@@ -415,8 +415,9 @@ class BatchSolver:
     """Many independent 2D grids of uneven size advanced together (hydro_batch_* of the C ABI).
 
     shapes: sequence of (nx, ny); every grid is its own unit square with its own CFL dt.
-    tile: (bx, by) of the batch kernels, default (32, 8); (bx, 1) selects row tiles, which march
-    along y through `march` rows per work item (default 32).
+    tile: (bx, by) of the batch kernels; (bx, 1) selects row tiles, which march along y through
+    `march` rows per work item (FP32: strips of 60 columns whatever bx, the default, the rows
+    chosen from the grids unless named; FP64: default 32 rows, the default tile is (32, 8)).
     The packed state is a tensor of shape (4, total_cells): plane k holds grid g's cells at
     [offsets[g], offsets[g+1]), x fastest.
     """

@@ -79,6 +79,18 @@ def test_narrow_grids_run_the_faster_kernel_with_the_same_result(shape, kernel):
     assert torch.equal(U, W)
 
 
+def test_host_stepping_on_a_narrow_grid():
+    """The last step's tiles run slab by slab there, as the strips do."""
+    shape = (29, 150, 151)
+    S = hydro.Solver(shape, 1.4, dtype=F32)
+    U = _state(shape)
+    host = U.cpu().pin_memory()
+    out = torch.empty_like(host).pin_memory()
+    done = S.step(U, 3)
+    assert S.step_host(torch.empty_like(U), host, out, 3) == done
+    assert torch.equal(out, U.cpu())
+
+
 @pytest.mark.parametrize("shape", [(512, 512), (1024, 1024), (2048, 2048), (4096, 4096), (300, 77),
                                    (64, 64, 64), (128, 128, 128), (160, 160, 160), (40, 36, 30)])
 def test_the_tuner_can_name_the_default(shape):
